@@ -55,7 +55,7 @@ SCHEDULERS_PER_SM = 4
 # signature and the SHA-256 of its sources.  When the built kernel differs,
 # the line says roofline.stale = true and drops traffic (the counters must
 # be taken again).
-TIMED_KERNEL = "_ZN3lxo11k_propagateILb0ELb0ELb0ELi256ELi8EEEvNS_10PropParamsE"   # k_propagate<0,0,0,256,8>
+TIMED_KERNEL = "_ZN3lxo11k_propagateILb0ELb0ELb0EEEvNS_10PropParamsE"   # k_propagate<0,0,0>
 KERNEL_SOURCES = ("paper_2203_14354_gb300/csrc/lxo_kernels.cu", "paper_2203_14354_gb300/csrc/lxo_internal.h")
 CAPTURED_KERNEL = {"registers": 32, "spill_stores": 538, "spill_loads": 616,
                    "sources_sha256": "1fa675c8893873eba0ba098175fb9ad1a31d29e08863aa4f1dad41da785a8a8a"}

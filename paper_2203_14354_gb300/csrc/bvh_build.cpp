@@ -15,6 +15,7 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <mutex>
 #include <thread>
 #include <vector>
 
@@ -56,7 +57,7 @@ struct TmpNode {
 
 // surface-area heuristic: cost of a triangle test relative to a node visit
 #ifndef LXO_SAH_CI
-#define LXO_SAH_CI 1.0
+#define LXO_SAH_CI 2.0
 #endif
 constexpr double kSahTriCost = LXO_SAH_CI;
 
@@ -319,6 +320,114 @@ Ref make_ref(const float* tri_v, uint32_t id)
     return r;
 }
 
+// Cells of the walk grid along the longest side of the scene.
+#ifndef LXO_GRID_CELLS
+#define LXO_GRID_CELLS 96
+#endif
+
+// The walk grid: cubic cells over the scene's bounding box and one cell
+// around it, x fastest.
+struct WalkGrid {
+    int n[3] = {0, 0, 0};
+    double org[3] = {0, 0, 0}, h = 0.0, pad = 0.0;
+    size_t cells() const { return (size_t)n[0] * n[1] * n[2]; }
+    size_t index(int i, int j, int k) const { return ((size_t)k * n[1] + j) * n[0] + i; }
+};
+
+template <class F>
+void parallel_for(uint32_t n_threads, size_t n, size_t grain, F&& body)   // body(first, last) over [0, n)
+{
+    std::atomic<size_t> next{0};
+    auto work = [&]() {
+        for (size_t i = next.fetch_add(grain); i < n; i = next.fetch_add(grain)) body(i, std::min(n, i + grain));
+    };
+    std::vector<std::thread> th;
+    for (uint32_t t = 1; t < std::min<size_t>(n_threads, (n + grain - 1) / grain); ++t) th.emplace_back(work);
+    work();
+    for (auto& t : th) t.join();
+}
+
+// Cells that triangle v may touch, each once: a triangle whose box (widened
+// by the pad) spans more than two cells along an axis is halved across its
+// longest edge until its parts' boxes do not.
+void touched_cells(const WalkGrid& g, const float* v, std::vector<uint32_t>& out)
+{
+    double t[64][3][3];   // parts still to do
+    int depth[64], m = 1;
+    for (int j = 0; j < 3; ++j)
+        for (int a = 0; a < 3; ++a) t[0][j][a] = v[3 * j + a];
+    depth[0] = 0;
+    out.clear();
+    while (m) {
+        --m;
+        double w[3][3];
+        memcpy(w, t[m], sizeof w);
+        const int d = depth[m];
+        int lo[3], hi[3], span = 0;
+        for (int a = 0; a < 3; ++a) {
+            const double l = std::min(w[0][a], std::min(w[1][a], w[2][a])) - g.pad - g.org[a];
+            const double u = std::max(w[0][a], std::max(w[1][a], w[2][a])) + g.pad - g.org[a];
+            lo[a] = std::min(std::max(0, (int)std::floor(l / g.h)), g.n[a] - 1);
+            hi[a] = std::min(std::max(0, (int)std::floor(u / g.h)), g.n[a] - 1);
+            span = std::max(span, hi[a] - lo[a]);
+        }
+        if (span > 1 && d < 48 && m + 2 <= 64) {
+            int e = 0;
+            double best = -1.0;
+            for (int k = 0; k < 3; ++k) {
+                double l2 = 0.0;
+                for (int a = 0; a < 3; ++a) l2 += (w[(k + 1) % 3][a] - w[k][a]) * (w[(k + 1) % 3][a] - w[k][a]);
+                if (l2 > best) { best = l2; e = k; }
+            }
+            const int p = e, q = (e + 1) % 3, r = (e + 2) % 3;
+            for (int a = 0; a < 3; ++a) {
+                const double mid = 0.5 * (w[p][a] + w[q][a]);
+                t[m][0][a] = w[p][a]; t[m][1][a] = mid; t[m][2][a] = w[r][a];
+                t[m + 1][0][a] = mid; t[m + 1][1][a] = w[q][a]; t[m + 1][2][a] = w[r][a];
+            }
+            depth[m] = depth[m + 1] = d + 1;
+            m += 2;
+            continue;
+        }
+        for (int k = lo[2]; k <= hi[2]; ++k)
+            for (int j = lo[1]; j <= hi[1]; ++j)
+                for (int i = lo[0]; i <= hi[0]; ++i) out.push_back((uint32_t)g.index(i, j, k));
+    }
+    std::sort(out.begin(), out.end());
+    out.erase(std::unique(out.begin(), out.end()), out.end());
+}
+
+// Skips (see Scene::walk_skip) from the occupied cells: for each octant of
+// directions, the edge of the largest empty cube of cells that starts at the
+// cell and extends that way is 1 + the smallest edge at its seven neighbours
+// that way; occupied and outer cells end it.
+void walk_skips(const WalkGrid& g, const std::vector<uint8_t>& occ, uint32_t n_threads, std::vector<uint8_t>& skip)
+{
+    const int nx = g.n[0], ny = g.n[1], nz = g.n[2];
+    skip.resize(8 * g.cells());
+    parallel_for(n_threads, 8, 1, [&](size_t oct, size_t) {
+        const int sx = oct & 1 ? -1 : 1, sy = oct & 2 ? -1 : 1, sz = oct & 4 ? -1 : 1;   // bit set: towards smaller coordinates
+        auto at = [&](int i, int j, int k) -> uint8_t& { return skip[8 * g.index(i, j, k) + oct]; };
+        auto edge = [&](int i, int j, int k) -> int { const int v = at(i, j, k); return v == kCellOut ? 0 : v; };
+        for (int kk = 0; kk < nz; ++kk)
+            for (int jj = 0; jj < ny; ++jj)
+                for (int ii = 0; ii < nx; ++ii) {
+                    // from the far end of the octant backwards
+                    const int i = sx > 0 ? nx - 1 - ii : ii, j = sy > 0 ? ny - 1 - jj : jj, k = sz > 0 ? nz - 1 - kk : kk;
+                    if (i == 0 || i == nx - 1 || j == 0 || j == ny - 1 || k == 0 || k == nz - 1) {
+                        at(i, j, k) = kCellOut;
+                    } else if (occ[g.index(i, j, k)]) {
+                        at(i, j, k) = 0;
+                    } else {
+                        int m = 253;
+                        for (int q = 1; q < 8; ++q)
+                            m = std::min(m, edge(i + (q & 1 ? sx : 0), j + (q & 2 ? sy : 0), k + (q & 4 ? sz : 0)));
+                        at(i, j, k) = (uint8_t)(m + 1);
+                    }
+                }
+    });
+}
+
 }  // namespace
 
 int build_bvh(const float* tri_v, uint32_t nt, const int32_t* cluster_of, int n_clusters, uint32_t leaf_size,
@@ -422,8 +531,64 @@ int build_bvh(const float* tri_v, uint32_t nt, const int32_t* cluster_of, int n_
         if (e <= max_ext) main_refs.push_back(r);
         else split_refs(&tri_v[9ull * i], i, r.b, max_ext, 0, main_refs);
     }
+    // walk grid: the main-tree triangles again, each in every cell that it
+    // touches, by its part inside the cell (both widened by the pad, 1 % of a
+    // cell); left out (kept empty) if that takes more than kMaxGridRefs parts
+    WalkGrid wg;
+    std::vector<std::pair<uint32_t, Ref>> grid_refs;
+    const bool flat = !(scene_ext > 0.0f);
+    out->grid_h = flat ? 1.0 : (double)scene_ext / LXO_GRID_CELLS;
+    if (!flat) {
+        Box sb;
+        sb.reset();
+        for (uint64_t k = 0; k < 3ull * nt; ++k) sb.grow(&tri_v[3 * k]);
+        wg.h = out->grid_h;
+        wg.pad = std::max(0.01 * wg.h, 4.0 * (double)expand);
+        for (int a = 0; a < 3; ++a) {
+            wg.n[a] = std::max(1, (int)std::ceil(((double)sb.hi[a] - sb.lo[a]) / wg.h)) + 2;
+            wg.org[a] = out->grid_org[a] = (double)sb.lo[a] - wg.h;
+        }
+        std::vector<uint32_t> ids;
+        for (uint32_t i = 0; i < nt; ++i)
+            if (in_main[i]) ids.push_back(i);
+        std::mutex mu;
+        std::atomic<uint64_t> total{0};
+        parallel_for(n_threads, ids.size(), 256, [&](size_t q, size_t e) {
+            std::vector<uint32_t> cells;
+            std::vector<std::pair<uint32_t, Ref>> part;
+            for (; q < e && total.load() + part.size() <= kMaxGridRefs; ++q) {
+                const float* v = &tri_v[9ull * ids[q]];
+                touched_cells(wg, v, cells);
+                for (uint32_t c : cells) {
+                    const int ijk[3] = {(int)(c % wg.n[0]), (int)(c / wg.n[0] % wg.n[1]),
+                                        (int)(c / wg.n[0] / wg.n[1])};
+                    double lo[3], hi[3];
+                    for (int a = 0; a < 3; ++a) {
+                        lo[a] = wg.org[a] + ijk[a] * wg.h - wg.pad;
+                        hi[a] = wg.org[a] + (ijk[a] + 1) * wg.h + wg.pad;
+                    }
+                    Ref r;
+                    if (!clipped_box(v, lo, hi, r.b)) continue;
+                    for (int a = 0; a < 3; ++a) r.c[a] = 0.5f * (r.b.lo[a] + r.b.hi[a]);
+                    r.id = ids[q];
+                    part.push_back({c, r});
+                }
+            }
+            total += part.size();
+            std::lock_guard<std::mutex> lock(mu);
+            grid_refs.insert(grid_refs.end(), part.begin(), part.end());
+        });
+        if (total.load() > kMaxGridRefs) {
+            std::vector<std::pair<uint32_t, Ref>>().swap(grid_refs);
+            wg = WalkGrid();
+        }
+        std::sort(grid_refs.begin(), grid_refs.end(), [](const auto& x, const auto& y) {
+            return x.first < y.first || (x.first == y.first && x.second.id < y.second.id);
+        });
+    }
+    const uint64_t n_grid = grid_refs.size();
     const uint64_t n_main = main_refs.size();
-    const uint64_t n_refs = n_main + n_dup;
+    const uint64_t n_refs = n_main + n_dup + n_grid;
     if (n_refs >= (1ull << 28)) {
         snprintf(err, err_len, "build_bvh: %llu triangle records exceed 2^28", (unsigned long long)n_refs);
         return -1;
@@ -467,6 +632,7 @@ int build_bvh(const float* tri_v, uint32_t nt, const int32_t* cluster_of, int n_
                     refs[kc.cell_first[q] + fill[c][q]++] = rc;
                 }
         }
+        for (uint64_t k = 0; k < n_grid; ++k) refs[n_main + n_dup + k] = grid_refs[k].second;
     }
 
     // ---- trees ----------------------------------------------------------------
@@ -503,6 +669,24 @@ int build_bvh(const float* tri_v, uint32_t nt, const int32_t* cluster_of, int n_
         for (auto& t : th) t.join();
         cl_root[c] = kd_top(B, cell_root[c], kc.nu, 0, kc.nu, 0, kc.nv);
     }
+    std::vector<std::pair<uint32_t, int32_t>> grid_root;   // (cell, tmp node) of the occupied cells
+    {
+        std::vector<uint64_t> first;
+        for (uint64_t k = 0; k < n_grid; ++k)
+            if (k == 0 || grid_refs[k].first != grid_refs[k - 1].first) {
+                grid_root.push_back({grid_refs[k].first, -1});
+                first.push_back(k);
+            }
+        first.push_back(n_grid);
+        parallel_for(n_threads, grid_root.size(), 64, [&](size_t q, size_t e) {
+            for (; q < e; ++q) {
+                const uint32_t r = B.alloc();
+                B.build(r, (uint32_t)(n_main + n_dup + first[q]), (uint32_t)(first[q + 1] - first[q]), 0);
+                grid_root[q].second = (int32_t)r;
+            }
+        });
+        std::vector<std::pair<uint32_t, Ref>>().swap(grid_refs);
+    }
     const uint32_t n_tmp = B.n_nodes.load();
 
     // ---- layout: depth-first per tree, main tree first ------------------------
@@ -526,6 +710,7 @@ int build_bvh(const float* tri_v, uint32_t nt, const int32_t* cluster_of, int n_
     if (main_leaf) main_wrap = n_internal++;  // a one-leaf root node wraps a leaf main tree
     dfs(main_tmp);
     for (int c = 0; c < n_clusters; ++c) dfs(cl_root[c]);
+    for (const auto& r : grid_root) dfs(r.second);
     out->n_nodes = std::max(1u, n_internal);
     out->n_leaves = n_leaves;
     out->n_records = (uint32_t)n_refs;
@@ -559,7 +744,11 @@ int build_bvh(const float* tri_v, uint32_t nt, const int32_t* cluster_of, int n_
     };
     auto put_box = [&](float4* f, int slot, const Box& b) {
         for (int a = 0; a < 3; ++a) {
-            const float lo = b.lo[a] - expand, hi = b.hi[a] + expand;
+            // in grid space, rounded outwards
+            const float lo = std::nextafter((float)(((double)b.lo[a] - expand - out->grid_org[a]) / out->grid_h),
+                                            -INFINITY);
+            const float hi = std::nextafter((float)(((double)b.hi[a] + expand - out->grid_org[a]) / out->grid_h),
+                                            INFINITY);
             if (slot == 0) { f[a].x = lo; f[a].y = hi; }
             else { f[a].z = lo; f[a].w = hi; }
         }
@@ -606,6 +795,23 @@ int build_bvh(const float* tri_v, uint32_t nt, const int32_t* cluster_of, int n_
         cell_off += (uint32_t)kc.cell_count.size();
     }
     out->n_cells = cell_off;
+    try {
+        if (wg.cells()) {
+            std::vector<uint8_t> occ(wg.cells(), 0);
+            out->walk_ref.assign(wg.cells(), kEmptyChild);
+            for (const auto& r : grid_root) {
+                occ[r.first] = 1;
+                out->walk_ref[r.first] = child_ref(r.second);
+            }
+            walk_skips(wg, occ, n_threads, out->walk_skip);
+            for (int a = 0; a < 3; ++a) out->walk_n[a] = wg.n[a];
+        }
+    } catch (...) {
+        free(nodes);
+        free_bvh(out);
+        snprintf(err, err_len, "build_bvh: out of host memory");
+        return -1;
+    }
     free(nodes);
     out->sah_cost = sah;
     out->build_seconds = std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();

@@ -42,6 +42,8 @@ struct lxo_ctx {
     float4* d_nodes = nullptr;
     float4* d_tris = nullptr;
     int32_t* d_cells = nullptr;
+    uint8_t* d_walk_skip = nullptr;
+    int32_t* d_walk_ref = nullptr;
     lxo::Scene scene{};
     unsigned long long* d_queue = nullptr;  // scratch: work-queue head
     int* d_err = nullptr;                   // scratch: device error word
@@ -100,6 +102,10 @@ void free_device_geometry(lxo_ctx* c)
     if (c->d_nodes) cudaFree(c->d_nodes);
     if (c->d_tris) cudaFree(c->d_tris);
     if (c->d_cells) cudaFree(c->d_cells);
+    if (c->d_walk_skip) cudaFree(c->d_walk_skip);
+    if (c->d_walk_ref) cudaFree(c->d_walk_ref);
+    c->d_walk_skip = nullptr;
+    c->d_walk_ref = nullptr;
     c->d_nodes = nullptr;
     c->d_tris = nullptr;
     c->d_cells = nullptr;
@@ -435,6 +441,13 @@ lxo_status lxo_build_bvh(lxo_ctx* c, const lxo_bvh_params* bp, lxo_bvh_info* inf
     if (e == cudaSuccess) e = cudaMemcpy(c->d_tris, b.tris, tb, cudaMemcpyHostToDevice);
     if (e == cudaSuccess && b.n_cells) e = cudaMemcpy(c->d_cells, b.cells, sizeof(int32_t) * b.n_cells,
                                                       cudaMemcpyHostToDevice);
+    const size_t wn = b.walk_ref.size();
+    if (e == cudaSuccess && wn) e = cudaMalloc(&c->d_walk_skip, 8 * wn);
+    if (e == cudaSuccess && wn) e = cudaMalloc(&c->d_walk_ref, sizeof(int32_t) * wn);
+    if (e == cudaSuccess && wn) e = cudaMemcpy(c->d_walk_skip, b.walk_skip.data(), 8 * wn,
+                                               cudaMemcpyHostToDevice);
+    if (e == cudaSuccess && wn) e = cudaMemcpy(c->d_walk_ref, b.walk_ref.data(), sizeof(int32_t) * wn,
+                                               cudaMemcpyHostToDevice);
     if (e != cudaSuccess) {
         lxo::free_bvh(&b);
         free_device_geometry(c);
@@ -462,6 +475,28 @@ lxo_status lxo_build_bvh(lxo_ctx* c, const lxo_bvh_params* bp, lxo_bvh_info* inf
         d.inv_cell = h.inv_cell;
         d.delta = expand;
         d.cells = c->d_cells + h.cells_offset;
+    }
+    for (int a = 0; a < 3; ++a)
+        for (int k = 0; k < lxo::kMaxClusters; ++k) {
+            const bool own = k < b.n_clusters && b.clusters[k].axis == a;
+            sc.layer_lo[a][k] = own ? b.clusters[k].slab_lo : INFINITY;
+            sc.layer_hi[a][k] = own ? b.clusters[k].slab_hi : -INFINITY;
+            if (own) sc.layer_axes |= 1u << a;
+        }
+    sc.grid_inv = (float)(1.0 / b.grid_h);
+    sc.grid_h = (float)b.grid_h;
+    for (int a = 0; a < 3; ++a) sc.grid_off[a] = (float)(-b.grid_org[a] / b.grid_h);
+    sc.walk_skip = c->d_walk_skip;
+    sc.walk_ref = c->d_walk_ref;
+    if (wn) {
+        for (int a = 0; a < 3; ++a) {
+            sc.walk_n[a] = b.walk_n[a];
+            sc.walk_max[a] = (float)b.walk_n[a] - 0.5f;
+        }
+        sc.walk_cells = (uint32_t)wn;
+        sc.walk_unit = (float)(b.grid_h / 64.0);
+        sc.walk_per_mm = (float)(64.0 / b.grid_h);
+        sc.walk_eps = (float)(0.002 * b.grid_h);
     }
     lxo::free_bvh(&b);
     c->info.n_tris = c->nt;

@@ -5,6 +5,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <vector>
+
 #include "../../include/lxo.h"
 
 namespace lxo {
@@ -22,7 +24,8 @@ constexpr int32_t kEmptyChild = INT32_MIN;  // empty layer cell or main tree
 // overflow, lxo_build_bvh bounds the depth), PMT channel out of range
 enum : int { kErrStack = 1, kErrChannel = 2, kErrBounds = 8 };
 
-// Node: 64 bytes, boxes of both children (x, y, z slabs) + child references.
+// Node: 64 bytes, boxes of both children (x, y, z slabs, in the scene's grid
+// space) + child references.
 //   f[0] = (c0.lo.x, c0.hi.x, c1.lo.x, c1.hi.x)
 //   f[1] = (c0.lo.y, c0.hi.y, c1.lo.y, c1.hi.y)
 //   f[2] = (c0.lo.z, c0.hi.z, c1.lo.z, c1.hi.z)
@@ -41,6 +44,17 @@ enum : int { kErrStack = 1, kErrChannel = 2, kErrBounds = 8 };
 // in-slab segment touches; other rays fall back to the cluster root.
 constexpr int kMaxClusters = 8;
 constexpr int kMaxCellsPerRay = 4;
+// walk grid: the skip of its outer cells, and the most parts of triangles it
+// may hold
+constexpr uint8_t kCellOut = 255;
+constexpr uint64_t kMaxGridRefs = 8u << 20;
+#ifndef LXO_SAFE_HOPS
+#define LXO_SAFE_HOPS 3
+#endif
+constexpr int kSafeHops = LXO_SAFE_HOPS;
+#ifndef LXO_POOL_KB
+#define LXO_POOL_KB 164
+#endif
 
 struct ClusterHost {
     int axis;
@@ -59,6 +73,10 @@ struct BvhHost {
     int32_t main_root = kEmptyChild;  // root of the tree over the non-cluster triangles
     int n_clusters = 0;
     ClusterHost clusters[kMaxClusters];
+    std::vector<uint8_t> walk_skip;   // walk grid (see Scene), empty if the scene has none
+    std::vector<int32_t> walk_ref;
+    int walk_n[3] = {0, 0, 0};
+    double grid_org[3] = {0, 0, 0}, grid_h = 1.0;   // grid space: (x - grid_org) / grid_h
     double sah_cost = 0.0, build_seconds = 0.0;
 };
 
@@ -113,6 +131,27 @@ struct Scene {
     int32_t main_root;     // kEmptyChild if every triangle is in a cluster
     int n_clusters;
     ClusterDev clusters[kMaxClusters];
+    // slabs of the clusters by axis (bit a of layer_axes: some cluster's
+    // normal is axis a); an entry of another axis or past n_clusters is an
+    // empty slab, which nothing meets
+    uint32_t layer_axes;
+    float layer_lo[3][kMaxClusters], layer_hi[3][kMaxClusters];
+    // Grid space: x * grid_inv + grid_off, cells of side grid_h (mm) as unit;
+    // the node boxes are in it.
+    float grid_inv, grid_h, grid_off[3];
+    // Walk grid over everything outside the planar clusters: cubic cells over
+    // the scene's box and one cell around it, x fastest.  walk_skip (NULL = no
+    // grid), 8 entries a cell, one for each octant of directions (bit a set:
+    // towards smaller coordinates along axis a): kCellOut an outer cell; 0 a
+    // cell with a sub-tree (walk_ref) over the parts of triangles inside; else
+    // k: the cube of k^3 cells from the cell on in that octant is empty.
+    const uint8_t* walk_skip;
+    const int32_t* walk_ref;
+    int walk_n[3];
+    uint32_t walk_cells;
+    float walk_max[3];   // coordinates within [0.5, walk_max] lie in a cell of the grid
+    float walk_eps;      // a nudge past a cell's side, mm
+    float walk_unit, walk_per_mm;   // unit of a clear distance kept in 16 bits (mm), and its inverse
 };
 
 // Emission-time profile: delay -tau ln u, tau = tau_s with probability f_s,
@@ -163,6 +202,7 @@ struct PropParams {
     uint32_t chunk;                    // photon ids per warp grab
     uint32_t blocks_per_sm;            // 0 = occupancy limit
     uint32_t block_threads;            // threads per CTA of the propagation kernel: 128 or 256 (0 = 256)
+    int slots, tally_stride;     // photon slots per CTA, floats of adjoint tallies per slot (set by the launch)
     unsigned long long* queue;   // scratch: work-queue head
     int* err;                    // scratch: device error word
 };

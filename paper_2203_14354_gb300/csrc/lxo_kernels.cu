@@ -2,13 +2,12 @@
 //
 //  * k_trace:          one ray per lane, closest hit (the geometry query alone).
 //  * k_sample_source:  first photon state from a source (one photon per lane).
-//  * k_propagate:      persistent kernel; each lane carries one photon from its
-//                      source to its fate (bulk absorption, Rayleigh, Fresnel /
-//                      TIR, reflectors, electrodes, photocathode).  A lane whose
-//                      photon died is refilled from a warp-local chunk of photon
-//                      ids (warp ballot + prefix popcount), chunks come from a
-//                      global atomic work queue: no lane idles while photons
-//                      remain.  Fate tallies live in shared memory per CTA;
+//  * k_propagate:      persistent kernel; the photons of a CTA wait in slots in
+//                      shared memory for one of four kinds of work (query of
+//                      the geometry, bulk event, surface event, tally and
+//                      rebirth), and each warp takes a batch of one kind (see
+//                      there).  Photon ids come from a global atomic work
+//                      queue; fate tallies live in shared memory per CTA;
 //                      per-channel counts and the time histogram use global
 //                      atomics.  Template builds <kStats, kAdjoint, kSpectral>
 //                      add traversal counters, the adjoint tallies, and a
@@ -20,10 +19,13 @@
 // the watertight test (Woop, Benthin & Wald, JCGT 2013); every operation is an
 // explicit round-to-nearest intrinsic so the compiler cannot contract or
 // reorder it.  Boxes are widened at build time and the box test uses a
-// relative slack, so the traversal visits every box that holds a candidate.
+// relative slack, so the traversal visits every box that holds a candidate;
+// the walk through the grid passes every cell that holds a part of one.
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
+
+#include <algorithm>
 
 #include "lxo_internal.h"
 
@@ -45,9 +47,16 @@ struct U4 {
     float u0, u1, u2, u3;
 };
 
-__device__ __forceinline__ uint4 philox4x32_10(uint4 c, uint2 k)
+#ifndef LXO_PHILOX_UNROLL
+#define LXO_PHILOX_UNROLL 10
+#endif
+#ifndef LXO_PHILOX_INLINE
+#define LXO_PHILOX_INLINE __forceinline__
+#endif
+constexpr int kPhiloxUnroll = LXO_PHILOX_UNROLL;
+static __device__ LXO_PHILOX_INLINE uint4 philox4x32_10(uint4 c, uint2 k)
 {
-#pragma unroll
+#pragma unroll kPhiloxUnroll
     for (int r = 0; r < 10; ++r) {
         uint32_t hi0 = __umulhi(0xD2511F53u, c.x), lo0 = 0xD2511F53u * c.x;
         uint32_t hi1 = __umulhi(0xCD9E8D57u, c.z), lo1 = 0xCD9E8D57u * c.z;
@@ -184,43 +193,39 @@ struct Hit {
     float t;
 };
 
-__device__ __forceinline__ float safe_inv(float d)
+// The reciprocal without IEEE rounding (1 ulp): the slab test is conservative
+// by the boxes' margin and the slack, so the hits are the same.
+__device__ __forceinline__ float fast_inv(float d)
 {
-    return __frcp_rn(fabsf(d) < 1e-20f ? copysignf(1e-20f, d) : d);
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(fabsf(d) < 1e-20f ? 1e-20f : d));
+    return r;
 }
 
-// lane cycles by phase of the photon loop (counting build): node loop, leaf
-// loop, traversal set-up (every entry, fresh or resumed), step draws,
-// interaction, refill (tallies and new photons)
+// Counting build: what one lane counts (warp-wide figures by lane 0).  Lane
+// cycles by phase of the photon loop, a warp's clock times the lanes at work:
+// node loop, leaf loop, traversal set-up (slots taken and read), random draws
+// and the next flight, interaction, refill (tallies, new photons).
 enum { kCycNode = 0, kCycLeaf, kCycBegin, kCycDraw, kCycFinish, kCycRefill, kCycPhases };
 
 struct Counters {
-    uint32_t nodes, leaves, tris;
-    uint32_t node_iters, leaf_iters;   // warp iterations of the node / leaf loops (counted by one lane)
-    unsigned long long trav_cycles;     // lane cycles inside the traversal
+    uint32_t steps, nodes, leaves, tris;
+    uint32_t node_iters, leaf_iters, batches, entries, walks, walk_iters;
+    uint32_t q_nodes, q_leaves;      // of the query in flight
+    unsigned long long loop_cycles, idle_cycles;
     unsigned long long cyc[kCycPhases];
 };
 
-__device__ __forceinline__ bool warp_leader()
-{
-    return (threadIdx.x & 31u) == (uint32_t)(__ffs(__activemask()) - 1);
-}
-
 // Leaf test of one leaf reference: every triangle of the leaf through the
 // exact watertight test, keeping (t, id) minimal in that order.
-template <bool kStats>
 __device__ __forceinline__ void test_leaf(const Scene& sc, const WRay& wr, int ref, uint32_t skip, float& bt,
-                                          uint32_t& best, uint32_t& best_rec, Counters& cnt, int* bounds_err)
+                                          uint32_t& best, uint32_t& best_rec, int* bounds_err)
 {
     const uint32_t enc = ~(uint32_t)ref;
     const uint32_t first = enc >> 3, count = (enc & 7u) + 1u;
     if (LXO_CHECK_BOUNDS && (uint64_t)first + count > sc.n_records) {
         atomicOr(bounds_err, kErrBounds);
         return;
-    }
-    if (kStats) {
-        cnt.leaves++;
-        cnt.tris += count;
     }
     for (uint32_t k = 0; k < count; ++k) {
         const float4* tr = sc.tris + 3 * (size_t)(first + k);
@@ -238,7 +243,44 @@ __device__ __forceinline__ void test_leaf(const Scene& sc, const WRay& wr, int r
     }
 }
 
-constexpr int kDone = INT32_MIN + 1;  // stack sentinel; never a valid leaf reference (< 2^28 records)
+// The next triangle of a leaf for a query of the photon pool, the leaf
+// reference moved on past it (0 after the last): origin and shear constants
+// from the query's slot, the closest triangle known by its record.  One
+// triangle a call, since the lanes of a warp hold leaves of different sizes
+// (all of a leaf at once ran 4.4 tests a call for 1.5 triangles a leaf).
+// The axes are not swapped for a negative dkz: the swap negates U, V, W, det
+// and T exactly, so every hit and t stays the same.
+__device__ __forceinline__ void slot_triangle(const Scene& sc, const float4* q, int kz, uint32_t skip, int& leaf,
+                                              float& bt, uint32_t& best_rec, int* bounds_err)
+{
+    const uint32_t enc = ~(uint32_t)leaf;
+    const uint32_t r = enc >> 3;
+    leaf = (enc & 7u) ? leaf - 7 : 0;   // (first + 1, count - 1): enc + 7
+    if (LXO_CHECK_BOUNDS && r >= sc.n_records) {
+        atomicOr(bounds_err, kErrBounds);
+        return;
+    }
+    const float4* tr = sc.tris + 3 * (size_t)r;
+    const float4 a = __ldg(tr + 0), b = __ldg(tr + 1), c = __ldg(tr + 2);
+    const float4 o = q[0], sh = q[4];
+    const int kx = kz == 2 ? 0 : kz + 1, ky = kz == 0 ? 2 : kz - 1;
+    const WRay wr{o.x, o.y, o.z, sh.x, sh.y, sh.z, kx, ky, kz};
+    const uint32_t id = __float_as_uint(c.y);
+    float t;
+    if (id != skip && wray_hit(wr, a, b, c, bt, t)) {
+        // ties go to the smallest triangle id
+        if (t < bt || best_rec == LXO_NO_HIT || id < __float_as_uint(__ldg(sc.tris + 3 * (size_t)best_rec + 2).y)) {
+            bt = t;
+            best_rec = r;
+        }
+    }
+}
+
+// Stack entries that are no leaf reference (those are above INT32_MIN + 6: < 2^28 records)
+constexpr int kDone = INT32_MIN + 1;  // bottom of the stack
+constexpr int kWalk = INT32_MIN + 2;  // back to the walk through the grid
+
+__device__ __forceinline__ bool is_leaf(int node) { return (uint32_t)node > (uint32_t)kWalk; }
 
 // Traversal state of one ray (its stack lives in a separate local
 // array of kStackSize entries).
@@ -253,32 +295,28 @@ struct TravState {
 
 // The per-ray constants of a query of ray (o, d) skipping triangle `skip`:
 // the watertight test's shear and the slab test's inverse direction.
-__device__ __forceinline__ void trav_setup(float3 o, float3 d, uint32_t skip, TravState& ts)
+__device__ __forceinline__ void trav_setup(const Scene& sc, float3 o, float3 d, uint32_t skip,
+                                           TravState& ts)
 {
     ts.wr = wray_setup(o, d);
-    ts.ix = safe_inv(d.x);
-    ts.iy = safe_inv(d.y);
-    ts.iz = safe_inv(d.z);
-    ts.oix = o.x * ts.ix;
-    ts.oiy = o.y * ts.iy;
-    ts.oiz = o.z * ts.iz;
+    ts.ix = fast_inv(d.x) * sc.grid_h;
+    ts.iy = fast_inv(d.y) * sc.grid_h;
+    ts.iz = fast_inv(d.z) * sc.grid_h;
+    ts.oix = fmaf(o.x, sc.grid_inv, sc.grid_off[0]) * ts.ix;
+    ts.oiy = fmaf(o.y, sc.grid_inv, sc.grid_off[1]) * ts.iy;
+    ts.oiz = fmaf(o.z, sc.grid_inv, sc.grid_off[2]) * ts.iz;
     ts.skip = skip;
 }
 
-// Enters the forest for a query with t in (0, tmax] (after trav_setup).
-// Planar clusters: a ray crossing the slab within a few grid cells starts at
-// those cells' sub-trees; any other ray meeting the slab at the cluster root.
-__device__ __forceinline__ void trav_enter(const Scene& sc, float3 o, float3 d, float tmax, TravState& ts,
-                                           int* stack)
+// Pushes the entries of the planar clusters in `mask` for a ray with t in
+// (0, tmax]: a ray crossing the slab within a few grid cells starts at those
+// cells' sub-trees; any other ray meeting the slab at the cluster root.
+__device__ __forceinline__ void enter_clusters(const Scene& sc, uint32_t mask, float3 o, float3 d, float tmax,
+                                               int* stack, int& sp)
 {
-    ts.bt = tmax;
-    ts.best = LXO_NO_HIT;
-    ts.best_rec = 0;
-    stack[0] = kDone;
-    int sp = 1;
-    for (int c = 0; c < sc.n_clusters; ++c) {
-        const ClusterDev& cl = sc.clusters[c];
-        const float oa = pick(cl.axis, o.x, o.y, o.z), ia = pick(cl.axis, ts.ix, ts.iy, ts.iz);
+    for (; mask; mask &= mask - 1) {
+        const ClusterDev& cl = sc.clusters[__ffs(mask) - 1];
+        const float oa = pick(cl.axis, o.x, o.y, o.z), ia = fast_inv(pick(cl.axis, d.x, d.y, d.z));
         const float ta = (cl.slab_lo - oa) * ia, tb = (cl.slab_hi - oa) * ia;
         const float tin = fmaxf(fminf(ta, tb), 0.0f), tout = fminf(fmaxf(ta, tb), tmax * kBoxSlack);
         if (!(tin <= tout)) continue;
@@ -305,6 +343,18 @@ __device__ __forceinline__ void trav_enter(const Scene& sc, float3 o, float3 d, 
         }
         stack[sp++] = cl.root;
     }
+}
+
+// Enters the forest for a query with t in (0, tmax] (after trav_setup).
+__device__ __forceinline__ void trav_enter(const Scene& sc, float3 o, float3 d, float tmax, TravState& ts,
+                                           int* stack)
+{
+    ts.bt = tmax;
+    ts.best = LXO_NO_HIT;
+    ts.best_rec = 0;
+    stack[0] = kDone;
+    int sp = 1;
+    enter_clusters(sc, (1u << sc.n_clusters) - 1u, o, d, tmax, stack, sp);
     ts.node = sc.main_root != kEmptyChild ? sc.main_root : stack[--sp];
     ts.leaf = 0;  // parked leaf (0 = none: reference 0 is an internal node, never a leaf)
     ts.sp = sp;
@@ -313,72 +363,66 @@ __device__ __forceinline__ void trav_enter(const Scene& sc, float3 o, float3 d, 
 __device__ __forceinline__ void trav_begin(const Scene& sc, float3 o, float3 d, uint32_t skip, float tmax,
                                            TravState& ts, int* stack)
 {
-    trav_setup(o, d, skip, ts);
+    trav_setup(sc, o, d, skip, ts);
     trav_enter(sc, o, d, tmax, ts, stack);
+}
+
+// One visit: the two children's boxes against the ray; descends into the
+// nearer child hit and pushes the other, or pops.
+__device__ __forceinline__ void node_visit(const Scene& sc, float ix, float iy, float iz, float oix, float oiy,
+                                           float oiz, float lim, int& node, int* stack, int& sp, int* err)
+{
+    if (LXO_CHECK_BOUNDS && (uint32_t)node >= sc.n_nodes) {
+        atomicOr(err, kErrBounds);
+        node = kDone;
+        sp = 1;
+        return;
+    }
+    const float4* nd = sc.nodes + 4 * (size_t)node;
+    const float4 nx = __ldg(nd + 0), ny = __ldg(nd + 1), nz = __ldg(nd + 2);
+    const int4 cr = __ldg(reinterpret_cast<const int4*>(nd + 3));
+    const float ax0 = fmaf(nx.x, ix, -oix), ax1 = fmaf(nx.y, ix, -oix);
+    const float ay0 = fmaf(ny.x, iy, -oiy), ay1 = fmaf(ny.y, iy, -oiy);
+    const float az0 = fmaf(nz.x, iz, -oiz), az1 = fmaf(nz.y, iz, -oiz);
+    const float bx0 = fmaf(nx.z, ix, -oix), bx1 = fmaf(nx.w, ix, -oix);
+    const float by0 = fmaf(ny.z, iy, -oiy), by1 = fmaf(ny.w, iy, -oiy);
+    const float bz0 = fmaf(nz.z, iz, -oiz), bz1 = fmaf(nz.w, iz, -oiz);
+    const float an = fmaxf(fmaxf(fminf(ax0, ax1), fminf(ay0, ay1)), fmaxf(fminf(az0, az1), 0.0f));
+    const float af = fminf(fminf(fmaxf(ax0, ax1), fmaxf(ay0, ay1)), fminf(fmaxf(az0, az1), lim));
+    const float bn = fmaxf(fmaxf(fminf(bx0, bx1), fminf(by0, by1)), fmaxf(fminf(bz0, bz1), 0.0f));
+    const float bf = fminf(fminf(fmaxf(bx0, bx1), fmaxf(by0, by1)), fminf(fmaxf(bz0, bz1), lim));
+    const bool ha = an <= af;
+    const bool hb = bn <= bf;   // every node has two children (see the builder)
+    const bool b_first = hb && !(ha && an <= bn);
+    const int near = b_first ? cr.y : cr.x;
+    if (ha && hb) {
+        // lxo_build_bvh rejects a forest whose depth plus the <= 33 entries
+        // the forest entry pushes could reach kStackSize, so this cannot
+        // fire; only the checked build keeps the test (in the normal build
+        // the never-taken exit cost 5 % of the time)
+        if (LXO_CHECK_BOUNDS && sp >= kStackSize) {
+            atomicOr(err, kErrStack);
+            node = kDone;
+            sp = 1;
+            return;
+        }
+        stack[sp++] = b_first ? cr.x : cr.y;
+    }
+    node = near;
+    if (!(ha || hb)) node = stack[--sp];
 }
 
 // "While-while" traversal with postponed leaves (Aila & Laine, HPG 2009): a
 // lane that reaches a leaf parks it and keeps descending until every active
 // lane of the warp holds a leaf; then the warp tests leaves together.
-// Runs the query to completion, or with kYield until the end of the first
-// leaf phase after which some lane of the warp has finished its query: the
-// lanes still tracing then leave with a resumable state (node >= 0, no
-// parked leaf), so that the finished ones can take their next ray (dynamic
-// ray fetch, after Aila & Laine).
-template <bool kStats, bool kYield = false>
-__device__ void trav_run(const Scene& sc, TravState& ts, int* stack, int* err, Counters& cnt)
+__device__ void trav_run(const Scene& sc, TravState& ts, int* stack, int* err)
 {
     int node = ts.node, leaf = ts.leaf, sp = ts.sp;
     float bt = ts.bt;
     uint32_t best = ts.best, best_rec = ts.best_rec;
-    long long tq = kStats ? clock64() : 0;
     while (true) {
         while (node >= 0) {
-            if (kStats) {
-                cnt.nodes++;
-                if (warp_leader()) cnt.node_iters++;
-            }
-            if (LXO_CHECK_BOUNDS && (uint32_t)node >= sc.n_nodes) {
-                atomicOr(err, kErrBounds);
-                node = kDone;
-                sp = 1;
-                break;
-            }
-            const float4* nd = sc.nodes + 4 * (size_t)node;
-            const float4 nx = __ldg(nd + 0), ny = __ldg(nd + 1), nz = __ldg(nd + 2);
-            const int4 cr = __ldg(reinterpret_cast<const int4*>(nd + 3));
-            const float lim = bt * kBoxSlack;
-            const float ax0 = fmaf(nx.x, ts.ix, -ts.oix), ax1 = fmaf(nx.y, ts.ix, -ts.oix);
-            const float ay0 = fmaf(ny.x, ts.iy, -ts.oiy), ay1 = fmaf(ny.y, ts.iy, -ts.oiy);
-            const float az0 = fmaf(nz.x, ts.iz, -ts.oiz), az1 = fmaf(nz.y, ts.iz, -ts.oiz);
-            const float bx0 = fmaf(nx.z, ts.ix, -ts.oix), bx1 = fmaf(nx.w, ts.ix, -ts.oix);
-            const float by0 = fmaf(ny.z, ts.iy, -ts.oiy), by1 = fmaf(ny.w, ts.iy, -ts.oiy);
-            const float bz0 = fmaf(nz.z, ts.iz, -ts.oiz), bz1 = fmaf(nz.w, ts.iz, -ts.oiz);
-            const float an = fmaxf(fmaxf(fminf(ax0, ax1), fminf(ay0, ay1)), fmaxf(fminf(az0, az1), 0.0f));
-            const float af = fminf(fminf(fmaxf(ax0, ax1), fmaxf(ay0, ay1)), fminf(fmaxf(az0, az1), lim));
-            const float bn = fmaxf(fmaxf(fminf(bx0, bx1), fminf(by0, by1)), fmaxf(fminf(bz0, bz1), 0.0f));
-            const float bf = fminf(fminf(fmaxf(bx0, bx1), fmaxf(by0, by1)), fminf(fmaxf(bz0, bz1), lim));
-            const bool ha = an <= af;
-            const bool hb = bn <= bf;   // every node has two children (see the builder)
-            if (!ha && !hb) {
-                node = stack[--sp];
-            } else {
-                const bool a_first = ha && (!hb || an <= bn);
-                node = a_first ? cr.x : cr.y;
-                if (ha && hb) {
-                    // lxo_build_bvh rejects a forest whose depth plus the <= 33
-                    // entries trav_begin pushes could reach kStackSize, so this
-                    // cannot fire; only the checked build keeps the test (in the
-                    // normal build the never-taken exit cost 5 % of the time)
-                    if (LXO_CHECK_BOUNDS && sp >= kStackSize) {
-                        atomicOr(err, kErrStack);
-                        node = kDone;
-                        sp = 1;
-                        break;
-                    }
-                    stack[sp++] = a_first ? cr.y : cr.x;
-                }
-            }
+            node_visit(sc, ts.ix, ts.iy, ts.iz, ts.oix, ts.oiy, ts.oiz, bt * kBoxSlack, node, stack, sp, err);
             if (node < 0 && node != kDone && leaf == 0) {
                 leaf = node;
                 node = stack[--sp];
@@ -389,27 +433,15 @@ __device__ void trav_run(const Scene& sc, TravState& ts, int* stack, int* err, C
             leaf = node;
             node = stack[--sp];
         }
-        if (kStats) {
-            const long long t1 = clock64();
-            cnt.cyc[kCycNode] += (unsigned long long)(t1 - tq);
-            tq = t1;
-        }
         while (leaf != 0) {
-            if (kStats && warp_leader()) cnt.leaf_iters++;
-            test_leaf<kStats>(sc, ts.wr, leaf, ts.skip, bt, best, best_rec, cnt, err);
+            test_leaf(sc, ts.wr, leaf, ts.skip, bt, best, best_rec, err);
             leaf = 0;
             if (node < 0 && node != kDone) {
                 leaf = node;
                 node = stack[--sp];
             }
         }
-        if (kStats) {
-            const long long t1 = clock64();
-            cnt.cyc[kCycLeaf] += (unsigned long long)(t1 - tq);
-            tq = t1;
-        }
         if (node == kDone) break;
-        if (kYield && __activemask() != FULL_MASK) break;   // a lane finished (or was not tracing)
     }
     ts.node = node;
     ts.leaf = leaf;
@@ -424,55 +456,12 @@ __device__ __forceinline__ Hit trav_result(const TravState& ts)
     return Hit{ts.best, ts.best_rec, ts.best == LXO_NO_HIT ? INFINITY : ts.bt};
 }
 
-// State of a query between two entries to the traversal: node == kDone once
-// it has finished (best, best_rec and bt then hold the hit).
-struct TravResume {
-    float bt;
-    uint32_t best, best_rec;
-    int node, sp;
-};
-
-// One entry to the traversal for the photon loop: a query whose state says
-// kDone is new and enters the forest with t in (0, tmax]; any other resumes.
-// The per-ray constants are recomputed at every entry from (o, d): the warp
-// computes them anyway for its lanes that start a query, and they are not
-// kept in registers while the warp does its interactions.
-template <bool kStats>
-__device__ void trav_step(const Scene& sc, float3 o, float3 d, uint32_t skip, float tmax, TravResume& tr,
-                          int* stack, int* err, Counters& cnt)
-{
-    const long long t0 = kStats ? clock64() : 0;
-    TravState ts;
-    trav_setup(o, d, skip, ts);
-    if (tr.node == kDone) {
-        trav_enter(sc, o, d, tmax, ts, stack);
-    } else {
-        ts.bt = tr.bt;
-        ts.best = tr.best;
-        ts.best_rec = tr.best_rec;
-        ts.node = tr.node;
-        ts.leaf = 0;
-        ts.sp = tr.sp;
-    }
-    if (kStats) cnt.cyc[kCycBegin] += (unsigned long long)(clock64() - t0);
-    trav_run<kStats, true>(sc, ts, stack, err, cnt);
-    if (kStats) cnt.trav_cycles += (unsigned long long)(clock64() - t0);
-    tr.bt = ts.bt;
-    tr.best = ts.best;
-    tr.best_rec = ts.best_rec;
-    tr.node = ts.node;
-    tr.sp = ts.sp;
-}
-
-template <bool kStats>
-__device__ Hit closest_hit(const Scene& sc, float3 o, float3 d, uint32_t skip, float tmax, int* err, Counters& cnt)
+__device__ Hit closest_hit(const Scene& sc, float3 o, float3 d, uint32_t skip, float tmax, int* err)
 {
     TravState ts;
     int stack[kStackSize];
-    const long long t0 = kStats ? clock64() : 0;
     trav_begin(sc, o, d, skip, tmax, ts, stack);
-    if (kStats) cnt.cyc[kCycBegin] += (unsigned long long)(clock64() - t0);
-    trav_run<kStats>(sc, ts, stack, err, cnt);
+    trav_run(sc, ts, stack, err);
     return trav_result(ts);
 }
 
@@ -484,8 +473,7 @@ __global__ void k_trace(const Scene sc, const float* __restrict__ org, const flo
     if (i >= n) return;
     const float3 o = f3(org[3 * i], org[3 * i + 1], org[3 * i + 2]);
     const float3 d = f3(dir[3 * i], dir[3 * i + 1], dir[3 * i + 2]);
-    Counters cnt{};
-    const Hit h = closest_hit<false>(sc, o, d, skip ? skip[i] : LXO_NO_HIT, tmax ? tmax[i] : INFINITY, err, cnt);
+    const Hit h = closest_hit(sc, o, d, skip ? skip[i] : LXO_NO_HIT, tmax ? tmax[i] : INFINITY, err);
     hit[i] = h.id;
     t[i] = h.t;
 }
@@ -590,6 +578,7 @@ __device__ Photon make_event_photon(const PropParams& p, uint64_t idx)
     } else {
         ph.pos = f3(ev.center[0], ev.center[1], ev.center[2]);
         if (ev.kind == LXO_SRC_BALL) {
+#pragma unroll 1
             for (int tr = 0; tr < kMaxTries; ++tr) {
                 const U4 w = draw4(p.seed, ph.pid, kSourceStep, 1 + tr);
                 const float x = ev.radius * (2.0f * w.u0 - 1.0f), y = ev.radius * (2.0f * w.u1 - 1.0f),
@@ -604,7 +593,10 @@ __device__ Photon make_event_photon(const PropParams& p, uint64_t idx)
     return ph;
 }
 
-__device__ Photon make_photon(const PropParams& p, uint64_t idx)
+#ifndef LXO_MAKE_INLINE
+#define LXO_MAKE_INLINE
+#endif
+__device__ LXO_MAKE_INLINE Photon make_photon(const PropParams& p, uint64_t idx)
 {
     if (p.n_events) return make_event_photon(p, idx);
     const SourceDev& s = p.src;
@@ -635,6 +627,7 @@ __device__ Photon make_photon(const PropParams& p, uint64_t idx)
                     s.center[2] + u.u3 * (s.p1[2] - s.center[2]));
     } else if (s.kind == LXO_SRC_BALL) {
         ph.pos = f3(s.center[0], s.center[1], s.center[2]);
+#pragma unroll 1
         for (int tr = 0; tr < kMaxTries; ++tr) {
             const U4 w = draw4(p.seed, ph.pid, kSourceStep, 1 + tr);
             const float x = s.radius * (2.0f * w.u0 - 1.0f), y = s.radius * (2.0f * w.u1 - 1.0f),
@@ -646,6 +639,7 @@ __device__ Photon make_photon(const PropParams& p, uint64_t idx)
         }
     } else {
         ph.pos = f3(0.0f, 0.0f, s.z_min + u.u3 * (s.z_max - s.z_min));
+#pragma unroll 1
         for (int tr = 0; tr < kMaxTries; ++tr) {
             const U4 w = draw4(p.seed, ph.pid, kSourceStep, 1 + tr);
             float r = s.radius * sqrtf(w.u0), sa, ca;
@@ -665,15 +659,6 @@ __device__ Photon make_photon(const PropParams& p, uint64_t idx)
         }
     }
     return ph;
-}
-
-// Out of line, for the photon loop that resumes queries: inline, its
-// register demand spilled the traversal state that loop keeps across passes
-// (1.5 % faster out of line; the loop of whole steps is faster with it
-// inline).
-__device__ __noinline__ Photon make_photon_outlined(const PropParams& p, uint64_t idx)
-{
-    return make_photon(p, idx);
 }
 
 __global__ void k_sample_source(const __grid_constant__ PropParams p, float* pos, float* dir, float* pol,
@@ -825,59 +810,61 @@ __device__ __forceinline__ StepDraw begin_step(const PropParams& p, const Photon
     return sd;
 }
 
-template <bool kStats>
-__device__ __forceinline__ void step_histogram(const PropParams& p, const Photon& ph, uint32_t dn, uint32_t dl)
-{
-    // per-step histogram of node visits (8-wide bins) split by medium (0 vs other), and leaves
-    const int m = ph.medium == 0 ? 0 : 1;
-    atomicAdd(&p.out.stats[9 + 10 * m + min(dn / 8u, 8u)], 1ull);
-    atomicAdd(&p.out.stats[9 + 10 * m + 9], (unsigned long long)dl);
-}
 
-// Second half of a step: the interaction at the closest hit or in the bulk.
-// Returns -1 if the photon lives on, else its fate code (detail set to
-// channel / material / surface / triangle).
-// Adjoint tallies of one lane live in shared memory, tally k at tl[k * blockDim.x].
-constexpr int kAdjMaxK = 2 * (LXO_ADJ_MAX_MATERIALS + LXO_ADJ_MAX_SURFACES);
 
+
+// Second half of a step that met no surface: bulk absorption or Rayleigh
+// scattering at the sampled distance d_int (absorbed: the absorption distance
+// is the shorter one).  Returns -1 if the photon lives on, else its fate code
+// (detail set to the material).
 template <bool kAdjoint, bool kSpectral>
-__device__ int finish_step(const PropParams& p, Photon& ph, const StepDraw& sd, const Hit& h, int& detail,
-                           float* tl)
+__device__ __forceinline__ int bulk_event(const PropParams& p, Photon& ph, float d_int, bool absorbed, int& detail,
+                                          float* tl)
 {
-    const float d_abs = sd.d_abs, d_ray = sd.d_ray, d_int = fminf(d_abs, d_ray);
-    const U4 u = U4{0.0f, 0.0f, sd.u2, sd.u3};
+    if (isinf(d_int)) {
+        detail = -1;
+        return LXO_FATE_ESCAPED;
+    }
     const DevMaterial& mt = p.mat[ph.medium];
     const int ms = kAdjoint ? p.adj_mat_slot[ph.medium] : -1;
-    if (h.id == LXO_NO_HIT) {
-        if (isinf(d_int)) {
-            detail = -1;
-            return LXO_FATE_ESCAPED;
-        }
-        ph.pos = ph.pos + d_int * ph.dir;
-        ph.time += d_int * n_over_c_at<kSpectral>(mt, ph.wl);
-        if (kAdjoint && ms >= 0) tl[(2 * ms) * blockDim.x] += d_int;
-        if (d_abs <= d_ray) {
-            detail = ph.medium;
-            return LXO_FATE_BULK_ABS;
-        }
-        if (kAdjoint && ms >= 0) tl[(2 * ms + 1) * blockDim.x] += 1.0f;
-        rayleigh(ph, p.seed);
-        ph.last = LXO_NO_HIT;
-        return -1;
+    ph.pos = ph.pos + d_int * ph.dir;
+    ph.time += d_int * n_over_c_at<kSpectral>(mt, ph.wl);
+    if (kAdjoint && ms >= 0) tl[2 * ms] += d_int;
+    if (absorbed) {
+        detail = ph.medium;
+        return LXO_FATE_BULK_ABS;
     }
+    if (kAdjoint && ms >= 0) tl[2 * ms + 1] += 1.0f;
+    rayleigh(ph, p.seed);
+    ph.last = LXO_NO_HIT;
+    return -1;
+}
+
+// Second half of a step that met triangle record `rec` at distance t: the
+// interaction with its surface.  Returns -1 if the photon lives on, else its
+// fate code (detail set to channel / surface / triangle).
+template <bool kAdjoint, bool kSpectral>
+__device__ __forceinline__ int surface_event(const PropParams& p, Photon& ph, float t, uint32_t rec, int& detail,
+                                             float* tl)
+{
+    const DevMaterial& mt = p.mat[ph.medium];
+    const int ms = kAdjoint ? p.adj_mat_slot[ph.medium] : -1;
     const float3 o_ray = ph.pos;
-    ph.pos = ph.pos + h.t * ph.dir;
-    ph.time += h.t * n_over_c_at<kSpectral>(mt, ph.wl);
-    if (kAdjoint && ms >= 0) tl[(2 * ms) * blockDim.x] += h.t;
+    ph.pos = ph.pos + t * ph.dir;
+    ph.time += t * n_over_c_at<kSpectral>(mt, ph.wl);
+    if (kAdjoint && ms >= 0) tl[2 * ms] += t;
     // geometric normal and attributes of the triangle hit (record in leaf order)
-    if (LXO_CHECK_BOUNDS && h.rec >= p.sc.n_records) {
+    if (LXO_CHECK_BOUNDS && rec >= p.sc.n_records) {
         atomicOr(p.err, kErrBounds);
-        detail = (int)h.id;
+        detail = -1;
         return LXO_FATE_GEOM_ERR;
     }
-    const float4* tr = p.sc.tris + 3 * (size_t)h.rec;
+    const float4* tr = p.sc.tris + 3 * (size_t)rec;
     const float4 va = __ldg(tr + 0), vb = __ldg(tr + 1), vc = __ldg(tr + 2);
+    const uint32_t id = __float_as_uint(vc.y);
     const uint2 at = make_uint2(__float_as_uint(vc.z), __float_as_uint(vc.w));
+    // the step's first draw again (its first two uniforms gave the distances)
+    const U4 u = draw4(p.seed, ph.pid, ph.step, 0);
     const float3 e1 = f3(va.w - va.x, vb.x - va.y, vb.y - va.z);
     const float3 e2 = f3(vb.z - va.x, vb.w - va.y, vc.x - va.z);
     const float3 ng = normalize(cross(e1, e2));
@@ -886,16 +873,16 @@ __device__ int finish_step(const PropParams& p, Photon& ph, const StepDraw& sd, 
     const uint32_t sid = at.x >> 16;
     const int from = forward ? mi : mo, to = forward ? mo : mi;
     const float3 Nf = forward ? (-1.0f) * ng : ng;
-    ph.last = h.id;
+    ph.last = id;
     if (sid == LXO_SURF_NONE) {
         if (from != ph.medium || to >= p.n_mat) {
-            detail = (int)h.id;
+            detail = (int)id;
             return LXO_FATE_GEOM_ERR;
         }
         const bool refl = dielectric(ph, Nf, n_at<kSpectral>(p.mat[from], ph.wl), n_at<kSpectral>(p.mat[to], ph.wl),
                                       u.u2);
         if (!refl) ph.medium = to;
-        spawn_offset(ph, o_ray, h.t, Nf, refl ? 1.0f : -1.0f);
+        spawn_offset(ph, o_ray, t, Nf, refl ? 1.0f : -1.0f);
         return -1;
     }
     const DevSurface& sf = p.surf[sid];
@@ -907,7 +894,7 @@ __device__ int finish_step(const PropParams& p, Photon& ph, const StepDraw& sd, 
         const int ch = (int)at.y;
         if (ch < 0 || ch >= p.n_chan) {
             atomicOr(p.err, kErrChannel);
-            detail = (int)h.id;
+            detail = (int)id;
             return LXO_FATE_GEOM_ERR;
         }
         detail = ch;
@@ -921,73 +908,120 @@ __device__ int finish_step(const PropParams& p, Photon& ph, const StepDraw& sd, 
             detail = (int)sid;
             return LXO_FATE_SURF_ABS;
         }
-        if (kAdjoint && ss >= 0) tl[base_k * blockDim.x] += 1.0f;
+        if (kAdjoint && ss >= 0) tl[base_k] += 1.0f;
         specular = u.u3 < sf.spec;
     } else if (sf.type == LXO_SURF_ELECTRODE_T) {
         if (u.u2 < sf.T) {
             if (from != ph.medium || to >= p.n_mat) {
-                detail = (int)h.id;
+                detail = (int)id;
                 return LXO_FATE_GEOM_ERR;
             }
-            if (kAdjoint && ss >= 0) tl[base_k * blockDim.x] += 1.0f;
+            if (kAdjoint && ss >= 0) tl[base_k] += 1.0f;
             ph.medium = to;
-            spawn_offset(ph, o_ray, h.t, Nf, -1.0f);
+            spawn_offset(ph, o_ray, t, Nf, -1.0f);
             return -1;
         }
         if (!(u.u3 < sf.Rw)) {
             detail = (int)sid;
             return LXO_FATE_SURF_ABS;
         }
-        if (kAdjoint && ss >= 0) tl[(base_k + 1) * blockDim.x] += 1.0f;
+        if (kAdjoint && ss >= 0) tl[base_k + 1] += 1.0f;
         specular = draw4(p.seed, ph.pid, ph.step, 1).u3 < sf.wspec;
     } else {
-        detail = (int)h.id;
+        detail = (int)id;
         return LXO_FATE_GEOM_ERR;
     }
     if (specular)
         mirror(ph, Nf);
     else
         lambert(ph, Nf, p.seed);
-    spawn_offset(ph, o_ray, h.t, Nf, 1.0f);
+    spawn_offset(ph, o_ray, t, Nf, 1.0f);
     return -1;
-}
-
-// One whole step in one pass (draws, closest hit, interaction), for the
-// builds whose warps wait for their slowest query.
-template <bool kStats, bool kAdjoint, bool kSpectral>
-__device__ int photon_step(const PropParams& p, Photon& ph, int& detail, Counters& cnt, float* tl)
-{
-    const long long cd = kStats ? clock64() : 0;
-    const StepDraw sd = begin_step<kSpectral>(p, ph);
-    const long long c0 = kStats ? clock64() : 0;
-    if (kStats) cnt.cyc[kCycDraw] += (unsigned long long)(c0 - cd);
-    const uint32_t n0 = kStats ? cnt.nodes : 0, l0 = kStats ? cnt.leaves : 0;
-    const Hit h = closest_hit<kStats>(p.sc, ph.pos, ph.dir, ph.last, fminf(sd.d_abs, sd.d_ray), p.err, cnt);
-    if (kStats) {
-        cnt.trav_cycles += (unsigned long long)(clock64() - c0);
-        step_histogram<kStats>(p, ph, cnt.nodes - n0, cnt.leaves - l0);
-    }
-    const long long cf = kStats ? clock64() : 0;
-    const int fate = finish_step<kAdjoint, kSpectral>(p, ph, sd, h, detail, tl);
-    if (kStats) cnt.cyc[kCycFinish] += (unsigned long long)(clock64() - cf);
-    return fate;
 }
 
 // ---------------------------------------------------------------------------
 // persistent propagation kernel
 // ---------------------------------------------------------------------------
-// Register budgets, as CTAs of 256 threads per SM: every flavour of the
-// kernel is built for both and the launch shape picks one.  On the
-// DARWIN-scale forward workload (GB300) 8 CTAs (32 registers, the SM's 2048
-// threads) hide more latency than 6 (40 registers, +1.4 % time), 5 (48,
-// +5.4 %) or 4 (64, +9.8 %) despite their spills; the adjoint build and the
-// small 50 cm TPC, whose BVH stays in L1, run faster with 48 registers.
-// Lanes refill as soon as one is idle.
-#ifndef LXO_REFILL_MIN
-#define LXO_REFILL_MIN 1
+// A pool of photons per CTA.  Each photon lives in a slot in shared memory and
+// waits there, between the parts of its steps, in one of five sets: ready (its
+// next flight is to be traced), ready to enter a planar layer, bulk event due,
+// surface event due, free (its fate to be tallied, a new photon to be made).
+// A warp looks at the sets, takes up to 32 slots of one, does that work for
+// them, and puts them into the sets of what comes next.  What bounds the loop
+// is issue slots times lanes at work: the loop this replaced kept a photon in
+// a lane for its whole life and ran every kind of work for the few lanes that
+// needed it (9.3 lanes of 32 per instruction, 210 instructions per photon
+// step of a warp; here 17.3 and 114).  The draws of the next step and its
+// flight's set-up belong to the batch that ends the step before, with all
+// lanes at work.
+// Flights that meet nothing need no query: the walk grid's empty cubes clear
+// them (over half of the DARWIN-scale mesh's steps), which pays only because
+// the lanes of the others are then filled with other photons.
+// Measured (1e8 photons on the DARWIN-scale mesh / 3e6 on the 50 cm TPC with
+// dispersion / 2e6 on the mesh without electrodes, GB300): 503 / 21.0 / 17.7
+// ms before, 359 / 13.5 / 12.2 ms now.
+// Launch shape: CTAs of kPoolThreads threads, kPoolCtas per SM.
+#ifndef LXO_POOL_THREADS
+#define LXO_POOL_THREADS 640
 #endif
-constexpr int kBudgetFull = 8;   // 32 registers
-constexpr int kBudgetWide = 5;   // 48 registers
+#ifndef LXO_POOL_CTAS
+#define LXO_POOL_CTAS 2
+#endif
+// a warp leaves the traversal once 1 / kLeaveDiv of its rays have finished
+#ifndef LXO_LEAVE_DIV
+#define LXO_LEAVE_DIV 2
+#endif
+#ifndef LXO_WALK_MIN
+#define LXO_WALK_MIN 8
+#endif
+#ifndef LXO_NODE_MIN
+#define LXO_NODE_MIN 8
+#endif
+#ifndef LXO_STOP_DIV
+#define LXO_STOP_DIV 2
+#endif
+#ifndef LXO_BATCH_MIN
+#define LXO_BATCH_MIN 28
+#endif
+constexpr int kPoolThreads = LXO_POOL_THREADS, kPoolCtas = LXO_POOL_CTAS;
+constexpr int kPoolWarps = kPoolThreads / 32;
+constexpr int kMaxSlots = 1024;       // 32 columns of 32
+constexpr int kSlotF4 = 5;            // float4 per slot
+constexpr uint32_t kNoTri = 0x0FFFFFFFu;  // "no triangle" in 28 bits (ids stay below 2^28 - 1)
+constexpr uint32_t kPollLimit = 1u << 20;
+
+// Where a slot's photon waits.
+enum { kReady = 0, kReadyLayer, kBulk, kSurf, kFree, kSets };
+
+// A set of slots: bit j of word l stands for slot 32 j + l, so that lane l of
+// any warp takes slots of column l only, from its own word: no talk between
+// the lanes, no bank conflicts on the words or the slots (12 instructions;
+// packing the members of a set into the lanes by a prefix sum took 136 to
+// 194).  A slot leaves by atomicAnd, so none is taken twice and nothing waits.
+// `turn`: words are tried from that bit on, another for each warp.
+__device__ __forceinline__ int claim(uint32_t* set, uint32_t lanes, int turn, uint32_t lane)
+{
+    int slot = -1;
+    if ((lanes >> lane) & 1u) {
+        const uint32_t w = *(volatile uint32_t*)&set[lane];
+        if (w) {
+            const uint32_t r = __funnelshift_r(w, w, turn);
+            const int j = (__ffs(r) - 1 + turn) & 31;
+            if ((atomicAnd(&set[lane], ~(1u << j)) >> j) & 1u) slot = 32 * j + (int)lane;
+        }
+    }
+    __threadfence_block();   // a slot's contents are read after its bit was taken
+    return slot;
+}
+
+// At most n of the lanes in `lanes`.
+__device__ __forceinline__ uint32_t at_most(uint32_t lanes, int n)
+{
+    for (int m = __popc(lanes); m > n; --m) lanes &= lanes - 1u;
+    return lanes;
+}
+
+__device__ __forceinline__ void put(uint32_t* set, int slot) { atomicOr(&set[slot & 31], 1u << (slot >> 5)); }
 
 // Tally of one photon's fate: shared-memory fate counters, global per-channel
 // counts and arrival-time histogram, optional per-photon record and adjoint
@@ -1008,8 +1042,7 @@ __device__ __forceinline__ void tally(const PropParams& p, unsigned long long* s
         return;
     }
     if (kAdjoint && fate == LXO_FATE_DETECTED)
-        for (int k = 0; k < p.adj_k; ++k)
-            atomicAdd(&p.out.adjoint[row * p.adj_k + k], (double)tl[k * blockDim.x]);
+        for (int k = 0; k < p.adj_k; ++k) atomicAdd(&p.out.adjoint[row * p.adj_k + k], (double)tl[k]);
     atomicAdd(&s_f[fate], 1ull);
     atomicAdd(&s_f[7], (unsigned long long)ph.step);
     if (fate == LXO_FATE_BULK_ABS) atomicAdd(&s_f[LXO_FATES_FIXED + detail], 1ull);
@@ -1038,239 +1071,454 @@ __device__ __forceinline__ void tally(const PropParams& p, unsigned long long* s
     }
 }
 
-// Warp-uniform: makes sure the warp's chunk of photon ids is not empty,
-// taking the next p.chunk ids from the global work queue; false once the
-// queue is exhausted.
-__device__ __forceinline__ bool warp_chunk(const PropParams& p, uint32_t lane, unsigned long long& next,
-                                           unsigned long long& end, bool& exhausted)
+// Counting build: histogram of a step's node visits (8-wide bins) by medium
+// (0 or another), and its leaves.
+__device__ __forceinline__ void step_histogram(const PropParams& p, int medium, uint32_t dn, uint32_t dl)
 {
-    if (next < end) return true;
-    unsigned long long base = 0;
-    if (lane == 0) base = atomicAdd(p.queue, (unsigned long long)p.chunk);
-    base = __shfl_sync(FULL_MASK, base, 0);
-    if (base >= p.n) {
-        exhausted = true;
-        return false;
-    }
-    next = base;
-    end = min(base + p.chunk, (unsigned long long)p.n);
-    return true;
+    const int m = medium == 0 ? 0 : 1;
+    atomicAdd(&p.out.stats[9 + 10 * m + min(dn / 8u, 8u)], 1ull);
+    atomicAdd(&p.out.stats[9 + 10 * m + 9], (unsigned long long)dl);
 }
 
-// A photon in a warp's batch buffer: word j of slot k at o[j * kBatchN + k]
-// (consecutive lanes, consecutive banks).  Position, direction,
-// polarisation, id and, in the spectral build, the wavelength are kept;
-// medium and emission time follow from the id and the source when the
-// photon is taken, exactly as make_photon computes them (a smaller buffer
-// leaves more of the SM's memory to L1: 1.5 % faster than keeping all 13
-// words; the wavelength's Box-Muller draw is too dear to redo one lane at a
-// time).
-constexpr int kBatchN = 32;
-template <bool kSpectral>
-struct BatchSlot {
-    static constexpr int kWords = kSpectral ? 12 : 11;
-    static __device__ __forceinline__ void store(float* o, const Photon& q)
-    {
-        o[0 * kBatchN] = q.pos.x; o[1 * kBatchN] = q.pos.y; o[2 * kBatchN] = q.pos.z;
-        o[3 * kBatchN] = q.dir.x; o[4 * kBatchN] = q.dir.y; o[5 * kBatchN] = q.dir.z;
-        o[6 * kBatchN] = q.pol.x; o[7 * kBatchN] = q.pol.y; o[8 * kBatchN] = q.pol.z;
-        o[9 * kBatchN] = __uint_as_float((uint32_t)q.pid);
-        o[10 * kBatchN] = __uint_as_float((uint32_t)(q.pid >> 32));
-        if (kSpectral) o[11 * kBatchN] = q.wl;
-    }
-    static __device__ __forceinline__ Photon load(const float* o, const PropParams& p)
-    {
-        Photon q;
-        q.pos = f3(o[0 * kBatchN], o[1 * kBatchN], o[2 * kBatchN]);
-        q.dir = f3(o[3 * kBatchN], o[4 * kBatchN], o[5 * kBatchN]);
-        q.pol = f3(o[6 * kBatchN], o[7 * kBatchN], o[8 * kBatchN]);
-        q.pid = (uint64_t)__float_as_uint(o[9 * kBatchN]) | ((uint64_t)__float_as_uint(o[10 * kBatchN]) << 32);
-        if (p.n_events) {
-            const EventDev& ev = p.events[(uint32_t)(q.pid >> 32) - p.first_event];
-            q.medium = ev.medium;
-            q.time = ev.t0 + emission_delay(p, q.pid, ev.prof);
-        } else {
-            q.medium = p.src.medium;
-            q.time = p.src.t0 + emission_delay(p, q.pid, p.src.prof);
-        }
-        q.wl = kSpectral ? o[11 * kBatchN] : 0.0f;
-        q.last = LXO_NO_HIT;
-        q.step = 0;
-        return q;
-    }
-};
-
-// Persistent photon loop.  A lane whose photon reached its fate records its
-// tallies and takes the next photon id of its warp's chunk (ballot + prefix
-// popcount); chunks of p.chunk ids come from the global work-queue head.  A
-// lane refills as soon as it is idle (LXO_REFILL_MIN = 1: waiting for more
-// idle lanes measured slower).
-// Forward builds:
-// * Lanes do not wait for the slowest query of their warp: each pass of the
-//   loop traces until some lane has finished its query, and the unfinished
-//   queries resume in the next pass beside the fresh ones (dynamic ray
-//   fetch; on the DARWIN-scale mesh the lanes active in the node loop rose
-//   from 31 % to 45 % and in the leaf loop from 11 % to 20 %, 9 % less time).
-// * Photons are made a batch at a time: about one lane dies per pass, so
-//   when its shared-memory buffer is empty the warp makes the next kBatchN
-//   photons of its chunk, one per lane, and lanes that need a photon take
-//   the next ones from the buffer (7 % less time).
-// Adjoint builds keep whole steps and make photons lane by lane: with their
-// tallies the resumable loop was 4 % slower on the 50 cm TPC, whose tree
-// stays in L1.
-// Built for CTAs of kThreads = 256 (kBudget per SM) or 128 threads (twice as
-// many CTAs): the same registers per thread either way.
-template <bool kStats, bool kAdjoint, bool kSpectral, int kThreads, int kBudget>
-__global__ void __launch_bounds__(kThreads, kBudget * 256 / kThreads)
-    k_propagate(const __grid_constant__ PropParams p)
+// Distance at which a ray leaves the cube of k cells (an octant's) that starts
+// with its cell (x, y, z): in grid space, i = 1 / direction (large and positive
+// for a ray along a side), oi = origin * i.
+__device__ __forceinline__ float cube_exit(int x, int y, int z, float k, float ix, float iy, float iz, float oix,
+                                           float oiy, float oiz)
 {
-    constexpr bool kYield = !kAdjoint;
-    Counters cnt{};
-    uint32_t my_steps = 0, outer_iters = 0;
-    unsigned long long loop_cycles = 0;
+    const float tx = fmaf(k, fabsf(ix), fmaf((float)x, ix, fminf(ix, 0.0f) - oix));
+    const float ty = fmaf(k, fabsf(iy), fmaf((float)y, iy, fminf(iy, 0.0f) - oiy));
+    const float tz = fmaf(k, fabsf(iz), fmaf((float)z, iz, fminf(iz, 0.0f) - oiz));
+    return fminf(fminf(tx, ty), tz);
+}
+
+__device__ __forceinline__ uint32_t octant(float ix, float iy, float iz)
+{
+    return (__float_as_uint(ix) >> 31) | ((__float_as_uint(iy) >> 31) << 1) | ((__float_as_uint(iz) >> 31) << 2);
+}
+
+// How far a flight of length d from o along dir is clear by the walk grid's
+// empty cubes: true if all of it is; else `units` of walk_unit are clear,
+// kNoWalk if it starts outside the grid.
+constexpr uint32_t kNoWalk = 0xFFFFu;
+
+__device__ __forceinline__ bool clear_flight(const Scene& sc, float3 o, float3 dir, float d, uint32_t& units)
+{
+    units = kNoWalk;
+    if (!sc.walk_skip) return false;
+    const float gx = fmaf(o.x, sc.grid_inv, sc.grid_off[0]), gy = fmaf(o.y, sc.grid_inv, sc.grid_off[1]),
+                gz = fmaf(o.z, sc.grid_inv, sc.grid_off[2]);
+    const float ix = fast_inv(dir.x) * sc.grid_h, iy = fast_inv(dir.y) * sc.grid_h, iz = fast_inv(dir.z) * sc.grid_h;
+    const float ux = dir.x * sc.grid_inv, uy = dir.y * sc.grid_inv, uz = dir.z * sc.grid_inv;
+    const uint32_t oct = octant(ix, iy, iz);
+    float t = 0.0f;
+    bool clear = false;
+#pragma unroll 1
+    for (int hop = 0; hop < kSafeHops; ++hop) {
+        const int x = (int)fminf(fmaxf(fmaf(t, ux, gx), 0.5f), sc.walk_max[0]);
+        const int y = (int)fminf(fmaxf(fmaf(t, uy, gy), 0.5f), sc.walk_max[1]);
+        const int z = (int)fminf(fmaxf(fmaf(t, uz, gz), 0.5f), sc.walk_max[2]);
+        const uint32_t k = __ldg(&sc.walk_skip[8u * (uint32_t)((z * sc.walk_n[1] + y) * sc.walk_n[0] + x) + oct]);
+        if (k == kCellOut) {
+            if (hop == 0) return false;
+            clear = true;   // it has left the grid: nothing is ahead
+            break;
+        }
+        if (k == 0u) break;
+        t = fmaxf(cube_exit(x, y, z, (float)k, ix, iy, iz, gx * ix, gy * iy, gz * iz), t) + sc.walk_eps;
+        if (t > d) {
+            clear = true;
+            break;
+        }
+    }
+    units = min((uint32_t)(t * sc.walk_per_mm), kNoWalk - 1u);
+    return clear;
+}
+
+// One step of a query's walk through the grid: to the far side of the empty
+// cube ahead, or of an occupied cell, whose sub-tree is descended first.  The
+// triangles' parts reach over their cells by more than the nudge and the
+// rounding here.  The walk is over (the next stack entry follows) once it has
+// left the grid or passed the closest hit.
+__device__ __forceinline__ void walk_step(const Scene& sc, const float4* q, float ix, float iy, float iz, float oix,
+                                          float oiy, float oiz, float bt, float& t, int& node, int* stack, int& sp)
+{
+    const float4 a = q[0], b = q[1];
+    const int x = (int)fmaf(fmaf(t, b.x, a.x), sc.grid_inv, sc.grid_off[0]);
+    const int y = (int)fmaf(fmaf(t, b.y, a.y), sc.grid_inv, sc.grid_off[1]);
+    const int z = (int)fmaf(fmaf(t, b.z, a.z), sc.grid_inv, sc.grid_off[2]);
+    // (inside the grid by construction; the limit guards the memory)
+    const uint32_t c = min((uint32_t)((z * sc.walk_n[1] + y) * sc.walk_n[0] + x), sc.walk_cells - 1u);
+    const uint32_t k = __ldg(&sc.walk_skip[8u * c + octant(ix, iy, iz)]);
+    if (k == 0u) {
+        node = __ldg(&sc.walk_ref[c]);
+        stack[sp++] = kWalk;
+    }
+    t = fmaxf(cube_exit(x, y, z, fmaxf((float)k, 1.0f), ix, iy, iz, oix, oiy, oiz), t) + sc.walk_eps;
+    if (node == kWalk && (k == kCellOut || t > bt)) node = stack[--sp];
+}
+
+// Clusters whose slab the stretch of a ray with t in (0, tmax] may reach (bit
+// c); the slabs are wider than the rounding here.
+__device__ __forceinline__ uint32_t cluster_mask(const Scene& sc, float3 o, float3 d, float tmax)
+{
+    const float t = tmax * kBoxSlack;
+    const float ex = fmaf(t, d.x, o.x), ey = fmaf(t, d.y, o.y), ez = fmaf(t, d.z, o.z);
+    // (fminf and fmaxf skip the NaN of an unlimited ray with d = 0 along the axis)
+    const float l[3] = {fminf(o.x, ex), fminf(o.y, ey), fminf(o.z, ez)};
+    const float h[3] = {fmaxf(o.x, ex), fmaxf(o.y, ey), fmaxf(o.z, ez)};
+    uint32_t m = 0;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        if (!((sc.layer_axes >> a) & 1u)) continue;
+#pragma unroll
+        for (int c = 0; c < kMaxClusters; ++c)   // unused entries are empty slabs
+            m |= h[a] >= sc.layer_lo[a][c] && l[a] <= sc.layer_hi[a][c] ? 1u << c : 0u;
+    }
+    return m;
+}
+
+// A slot: five float4.
+//   [0] position, flight length (sign bit: absorption at its end) or hit distance
+//   [1] direction, a word: ready: axis kz | cluster mask << 2 | clear units << 16;  after the
+//       query: record hit (LXO_NO_HIT none);  free: fate (-1: no photon yet)
+//   [2] polarisation, time
+//   [3] id low, id high, step, medium << 28 | triangle left last
+//   [4] the watertight test's shear constants, wavelength
+__device__ __forceinline__ Photon load_slot(const float4* q)
+{
+    const float4 a = q[0], b = q[1], c = q[2], d = q[3];
+    Photon ph;
+    ph.pos = f3(a.x, a.y, a.z);
+    ph.dir = f3(b.x, b.y, b.z);
+    ph.pol = f3(c.x, c.y, c.z);
+    ph.time = c.w;
+    ph.wl = q[4].w;
+    ph.pid = (uint64_t)__float_as_uint(d.x) | ((uint64_t)__float_as_uint(d.y) << 32);
+    ph.step = __float_as_uint(d.z);
+    const uint32_t lm = __float_as_uint(d.w);
+    ph.medium = (int)(lm >> 28);
+    ph.last = (lm & kNoTri) == kNoTri ? LXO_NO_HIT : (lm & kNoTri);
+    return ph;
+}
+
+template <bool kStats, bool kAdjoint, bool kSpectral>
+__global__ void __launch_bounds__(kPoolThreads, kPoolCtas) k_propagate(const __grid_constant__ PropParams p)
+{
+    extern __shared__ float4 s_pool[];   // [p.slots] slots, then the adjoint tallies [p.slots][p.tally_stride]
     __shared__ unsigned long long s_f[kMaxFates];
-    __shared__ float s_tl[kAdjoint ? kAdjMaxK * kThreads : 1];
-    float* tl = kAdjoint ? &s_tl[threadIdx.x] : nullptr;
+    __shared__ uint32_t s_set[kSets][32];
+    __shared__ int s_live, s_dry;
     for (int i = threadIdx.x; i < p.n_fates; i += blockDim.x) s_f[i] = 0ull;
+    for (int i = threadIdx.x; i < kSets * 32; i += blockDim.x) {
+        const int rows = (p.slots - (i & 31) + 31) >> 5;   // slots of this column
+        s_set[i >> 5][i & 31] = (i >> 5) != kFree || rows <= 0 ? 0u : (rows >= 32 ? FULL_MASK : (1u << rows) - 1u);
+    }
+    for (int i = threadIdx.x; i < p.slots; i += blockDim.x) s_pool[kSlotF4 * i + 1].w = __int_as_float(-1);
+    if (threadIdx.x == 0) {
+        s_live = p.slots;
+        s_dry = 0;
+    }
     __syncthreads();
 
+    float* s_tally = reinterpret_cast<float*>(s_pool + kSlotF4 * p.slots);
     const uint32_t lane = threadIdx.x & 31u;
     const uint32_t lt_mask = (1u << lane) - 1u;
-    unsigned long long chunk_next = 0, chunk_end = 0;  // warp-uniform
-    bool exhausted = false;                             // warp-uniform
-    bool alive = false, pending = false;
-    int fate = 0, detail = -1;
-    Photon ph;
-    StepDraw sd;                 // the current step's draws
-    TravResume tr;               // its query (kDone: none in flight)
-    tr.node = kDone;
+    const int warp = threadIdx.x >> 5;
+    const int turn = warp & 31;
+    // the lane's query in flight: its slot (-1 none), closest hit so far and
+    // traversal state (kDone: not started); its stack in local memory
+    int slot = -1, node = kDone, sp = 1, kz = 0;
+    float bt = 0.0f, tw = 0.0f;
+    uint32_t rec = LXO_NO_HIT;
     int stack[kStackSize];
-    uint32_t n0 = 0, l0 = 0;     // counting build: node visits and leaves when the step began
-    using Slot = BatchSlot<kSpectral>;
-    __shared__ float s_batch[kYield ? (kThreads / 32) * Slot::kWords * kBatchN : 1];
-    float* batch = kYield ? &s_batch[(threadIdx.x >> 5) * Slot::kWords * kBatchN] : nullptr;
-    uint32_t batch_head = 0, batch_count = 0;   // warp-uniform: next buffered photon, photons buffered
+    uint32_t polls = 0;
+    Counters cnt{};
+    long long tick = kStats ? clock64() : 0;
+    // counting build: adds the warp's cycles since the last call, times the lanes at work
+    auto lap = [&](unsigned long long& sum, int lanes) {
+        if (!kStats) return;
+        const long long now = clock64();
+        if (lane == 0) {
+            sum += (unsigned long long)((now - tick) * lanes);
+            cnt.loop_cycles += (unsigned long long)((now - tick) * lanes);
+        }
+        tick = now;
+    };
 
     while (true) {
-        uint32_t need = __ballot_sync(FULL_MASK, !alive);
-        const int idle = __popc(need);
-        const long long cr = kStats ? clock64() : 0;
-        if (idle >= LXO_REFILL_MIN || idle == 32) {
-            if (pending) {
-                tally<kAdjoint>(p, s_f, ph, fate, detail, tl);
-                pending = false;
-            }
-            if constexpr (kYield) {
-                while (need && (batch_head < batch_count || !exhausted)) {
-                    if (batch_head == batch_count) {
-                        if (!warp_chunk(p, lane, chunk_next, chunk_end, exhausted)) break;
-                        const uint32_t make = min((uint32_t)(chunk_end - chunk_next), (uint32_t)kBatchN);
-                        if (lane < make) Slot::store(batch + lane, make_photon_outlined(p, chunk_next + lane));
-                        __syncwarp();
-                        chunk_next += make;
-                        batch_head = 0;
-                        batch_count = make;
-                    }
-                    const uint32_t take = min(batch_count - batch_head, (uint32_t)__popc(need));
-                    const uint32_t rank = __popc(need & lt_mask);
-                    if (((need >> lane) & 1u) && rank < take) {
-                        ph = Slot::load(batch + batch_head + rank, p);
-                        alive = true;
-                    }
-                    batch_head += take;
-                    __syncwarp();
-                    need = __ballot_sync(FULL_MASK, !alive);
-                }
-            }
-            while (!kYield && need && !exhausted) {
-                if (chunk_next >= chunk_end) {
-                    unsigned long long base = 0;
-                    if (lane == 0) base = atomicAdd(p.queue, (unsigned long long)p.chunk);
-                    base = __shfl_sync(FULL_MASK, base, 0);
-                    if (base >= p.n) {
-                        exhausted = true;
-                        break;
-                    }
-                    chunk_next = base;
-                    chunk_end = min(base + p.chunk, (unsigned long long)p.n);
-                }
-                const uint32_t avail = (uint32_t)(chunk_end - chunk_next);
-                const uint32_t take = min(avail, (uint32_t)__popc(need));
-                const uint32_t rank = __popc(need & lt_mask);
-                if (((need >> lane) & 1u) && rank < take) {
-                    ph = make_photon(p, chunk_next + rank);
-                    if (kAdjoint)
-                        for (int k = 0; k < p.adj_k; ++k) tl[k * kThreads] = 0.0f;
-                    alive = true;
-                }
-                chunk_next += take;
-                need = __ballot_sync(FULL_MASK, !alive);
-            }
+        uint32_t in[kSets];   // the lanes for which each set has a slot
+#pragma unroll
+        for (int k = 0; k < kSets; ++k) in[k] = __ballot_sync(FULL_MASK, *(volatile uint32_t*)&s_set[k][lane] != 0u);
+        const int live = __shfl_sync(FULL_MASK, *(volatile int*)&s_live, 0);
+        const uint32_t busy = __ballot_sync(FULL_MASK, slot >= 0);
+        // a batch: 32 lanes, fewer once the photons left do not fill all warps
+        const int width = min(32, (live + kPoolWarps - 1) / kPoolWarps);
+        const int full = width > LXO_BATCH_MIN ? LXO_BATCH_MIN : max(width, 1);
+        int stage;
+        if (__popc(in[kBulk]) >= full) stage = kBulk;
+        else if (__popc(in[kSurf]) >= full) stage = kSurf;
+        else if (__popc(in[kFree]) >= full) stage = kFree;
+        else if ((in[kReady] | in[kReadyLayer] | busy) != 0u) stage = kReady;
+        else if (in[kBulk]) stage = kBulk;
+        else if (in[kSurf]) stage = kSurf;
+        else if (in[kFree]) stage = kFree;
+        else {
+            // nothing to do here: other warps hold the photons left
+            if (live <= 0 || ++polls > kPollLimit) break;
+            __nanosleep(100);
+            lap(cnt.idle_cycles, 32);
+            continue;
         }
-        if (kStats) cnt.cyc[kCycRefill] += (unsigned long long)(clock64() - cr);
-        if (!__any_sync(FULL_MASK, alive || pending)) break;
-        if (kStats && lane == 0) outer_iters++;
-        const long long c0 = kStats ? clock64() : 0;
+
+        if (stage == kReady) {
+            // ---- traversal ------------------------------------------------
+            bool fresh = false;
+            const int room = width - __popc(busy);
+            if (room > 0) {
+                // queries that enter a layer's cells are taken apart from the others
+                const uint32_t fr = in[kReady] & ~busy, fl = in[kReadyLayer] & ~busy;
+                const int from = __popc(fl) > __popc(fr) ? kReadyLayer : kReady;
+                const uint32_t f = from == kReady ? fr : fl;
+                if (f) {
+                    const int t = claim(s_set[from], room < 32 ? at_most(f, room) : f, turn, lane);
+                    if (t >= 0) {
+                        slot = t;
+                        fresh = true;
+                    }
+                }
+            }
+            const int n0 = __popc(__ballot_sync(FULL_MASK, slot >= 0));
+            if (n0 == 0) continue;
+            const float4* q = s_pool + kSlotF4 * max(slot, 0);
+            float ix = 0.0f, iy = 0.0f, iz = 0.0f, oix = 0.0f, oiy = 0.0f, oiz = 0.0f;
+            uint32_t clusters = 0;
+            if (slot >= 0) {
+                const float4 a = q[0], b = q[1];
+                ix = fast_inv(b.x) * p.sc.grid_h;
+                iy = fast_inv(b.y) * p.sc.grid_h;
+                iz = fast_inv(b.z) * p.sc.grid_h;
+                oix = fmaf(a.x, p.sc.grid_inv, p.sc.grid_off[0]) * ix;
+                oiy = fmaf(a.y, p.sc.grid_inv, p.sc.grid_off[1]) * iy;
+                oiz = fmaf(a.z, p.sc.grid_inv, p.sc.grid_off[2]) * iz;
+                if (fresh) {
+                    const uint32_t kw = __float_as_uint(b.w);
+                    kz = (int)(kw & 3u);
+                    clusters = (kw >> 2) & 0xFFu;
+                    bt = fabsf(a.w);
+                    rec = LXO_NO_HIT;
+                    stack[0] = kDone;
+                    sp = 1;
+                    if (clusters)
+                        enter_clusters(p.sc, clusters, f3(a.x, a.y, a.z), f3(b.x, b.y, b.z), bt, stack, sp);
+                    // in the grid: the walk from where the flight is clear to;
+                    // else the main tree
+                    const uint32_t units = kw >> 16;
+                    tw = (float)units * p.sc.walk_unit;
+                    node = units != kNoWalk ? kWalk : p.sc.main_root;
+                    if (node == kEmptyChild) node = stack[--sp];
+                }
+            }
+            __syncwarp();
+            lap(cnt.cyc[kCycBegin], n0);
+            if (kStats && lane == 0) cnt.entries++;
+            int leaf = 0;   // parked leaf (0 = none: reference 0 is an internal node, never a leaf)
+            const int need = max(1, n0 / LXO_LEAVE_DIV);
+            const uint32_t skip = __float_as_uint(q[3].w) & kNoTri;
+            // Each pass runs the part of the traversal that most lanes wait
+            // for: a leaf's triangles, a step of the walk, a node.  A lane
+            // with a parked leaf walks or descends on until it meets the next.
+            while (true) {
+                if (leaf == 0 && is_leaf(node)) {
+                    leaf = node;
+                    node = stack[--sp];
+                }
+                if (node == kWalk && tw > bt) node = stack[--sp];
+                const int nw = __popc(__ballot_sync(FULL_MASK, node == kWalk));
+                const int nd = __popc(__ballot_sync(FULL_MASK, node >= 0));
+                const int nl = __popc(__ballot_sync(FULL_MASK, leaf != 0));
+                if (nl > 0 && nw < LXO_WALK_MIN && nd < LXO_NODE_MIN) {
+                    const int stop = nl / LXO_STOP_DIV;
+                    do {
+                        if (kStats && lane == 0) cnt.leaf_iters++;
+                        if (leaf != 0) {
+                            slot_triangle(p.sc, q, kz, skip, leaf, bt, rec, p.err);
+                            if (kStats) {
+                                cnt.q_leaves += leaf == 0;
+                                cnt.tris++;
+                            }
+                        }
+                    } while (__popc(__ballot_sync(FULL_MASK, leaf != 0)) > stop);
+                    lap(cnt.cyc[kCycLeaf], n0);
+                } else if (nw == 0 && nd == 0) {
+                    break;
+                } else if (nw >= nd) {
+                    const int stop = nw / LXO_STOP_DIV;
+                    do {
+                        if (kStats && lane == 0) cnt.walk_iters++;
+                        if (node == kWalk) {
+                            if (kStats) cnt.walks++;
+                            walk_step(p.sc, q, ix, iy, iz, oix, oiy, oiz, bt, tw, node, stack, sp);
+                        }
+                    } while (__popc(__ballot_sync(FULL_MASK, node == kWalk)) > stop);
+                    lap(cnt.cyc[kCycNode], n0);
+                } else {
+                    const int stop = nd / LXO_STOP_DIV;
+                    do {
+                        if (kStats && lane == 0) cnt.node_iters++;
+                        if (node >= 0) {
+                            if (kStats) cnt.q_nodes++;
+                            node_visit(p.sc, ix, iy, iz, oix, oiy, oiz, bt * kBoxSlack, node, stack, sp, p.err);
+                        }
+                    } while (__popc(__ballot_sync(FULL_MASK, node >= 0)) > stop);
+                    lap(cnt.cyc[kCycNode], n0);
+                }
+                if (n0 - __popc(__ballot_sync(FULL_MASK, node != kDone || leaf != 0)) >= need) break;
+            }
+            // a parked leaf goes back under the part of the query that is left
+            if (leaf != 0) {
+                stack[sp++] = node;
+                node = leaf;
+            }
+            const bool done = slot >= 0 && node == kDone;
+            if (done) {
+                float4* w = s_pool + kSlotF4 * slot;
+                if (rec != LXO_NO_HIT) w[0].w = bt;
+                w[1].w = __uint_as_float(rec);
+            }
+            if (kStats && done) {
+                step_histogram(p, (int)(__float_as_uint(q[3].w) >> 28), cnt.q_nodes, cnt.q_leaves);
+                cnt.nodes += cnt.q_nodes;
+                cnt.leaves += cnt.q_leaves;
+                cnt.q_nodes = cnt.q_leaves = 0;
+            }
+            __threadfence_block();
+            if (done) {
+                put(s_set[rec != LXO_NO_HIT ? kSurf : kBulk], slot);
+                slot = -1;
+            }
+            __syncwarp();
+            lap(cnt.cyc[kCycBegin], n0);
+            continue;
+        }
+
+        // ---- interactions, tallies and new photons ------------------------
+        const int want = stage == kFree ? min(width, (int)min(p.chunk, 32u)) : width;
+        const uint32_t lanes = stage == kBulk ? in[kBulk] : (stage == kSurf ? in[kSurf] : in[kFree]);
+        const int s = claim(s_set[stage], want < 32 ? at_most(lanes, max(want, 1)) : lanes, turn, lane);
+        const uint32_t members = __ballot_sync(FULL_MASK, s >= 0);
+        const int got = __popc(members);
+        if (got == 0) continue;
+        float4* q = s_pool + kSlotF4 * max(s, 0);
+        float* tl = kAdjoint ? s_tally + (size_t)max(s, 0) * p.tally_stride : nullptr;
+        Photon ph;
+        bool alive = false;
+        int fate = -1, detail = -1;
+        if (s >= 0) ph = load_slot(q);
+        if (stage == kFree) {
+            if (s >= 0) {
+                const int f = __float_as_int(q[1].w);
+                if (f >= 0) tally<kAdjoint>(p, s_f, ph, f, __float_as_int(q[0].w), tl);
+            }
+            unsigned long long base = p.n;
+            if (lane == 0 && !*(volatile int*)&s_dry) base = atomicAdd(p.queue, (unsigned long long)got);
+            base = __shfl_sync(FULL_MASK, base, 0);
+            const int avail = base < p.n ? (int)min((unsigned long long)got, (unsigned long long)p.n - base) : 0;
+            if (lane == 0 && avail < got) {
+                s_dry = 1;
+                atomicSub(&s_live, got - avail);
+            }
+            const int rank = __popc(members & lt_mask);
+            if (s >= 0 && rank < avail) {
+                ph = make_photon(p, base + rank);
+                if (kAdjoint)
+                    for (int k = 0; k < p.adj_k; ++k) tl[k] = 0.0f;
+                alive = true;
+            }
+        } else if (s >= 0) {
+            const float4 a = q[0], b = q[1];
+            if (stage == kBulk)
+                fate = bulk_event<kAdjoint, kSpectral>(p, ph, fabsf(a.w), (__float_as_uint(a.w) >> 31) != 0u, detail, tl);
+            else
+                fate = surface_event<kAdjoint, kSpectral>(p, ph, a.w, __float_as_uint(b.w), detail, tl);
+            ph.step++;
+            if (fate < 0 && ph.step >= p.max_steps) {
+                fate = LXO_FATE_TRUNCATED;
+                detail = -1;
+            }
+            alive = fate < 0;
+        }
+        if (kStats) {
+            if (lane == 0 && stage != kFree) {
+                cnt.steps += got;
+                cnt.batches++;
+            }
+            __syncwarp();
+            lap(cnt.cyc[stage == kFree ? kCycRefill : kCycFinish], got);
+        }
+        int to = -1;
         if (alive) {
-            // A step is the draws, a closest-hit query and the interaction.
-            // With kYield the query may span several passes of this loop: the
-            // warp leaves the traversal once one of its lanes has finished,
-            // and that lane interacts (or refills) and starts its next query
-            // while the others resume theirs.
-            bool stepped = true;
-            if constexpr (kYield) {
-                float tmax = 0.0f;
-                if (tr.node == kDone) {
-                    const long long cd = kStats ? clock64() : 0;
-                    sd = begin_step<kSpectral>(p, ph);
-                    tmax = fminf(sd.d_abs, sd.d_ray);
-                    if (kStats) {
-                        cnt.cyc[kCycDraw] += (unsigned long long)(clock64() - cd);
-                        n0 = cnt.nodes;
-                        l0 = cnt.leaves;
-                    }
-                }
-                trav_step<kStats>(p.sc, ph.pos, ph.dir, ph.last, tmax, tr, stack, p.err, cnt);
-                stepped = tr.node == kDone;
-                if (stepped) {
-                    if (kStats) step_histogram<kStats>(p, ph, cnt.nodes - n0, cnt.leaves - l0);
-                    const long long cf = kStats ? clock64() : 0;
-                    const Hit h{tr.best, tr.best_rec, tr.best == LXO_NO_HIT ? INFINITY : tr.bt};
-                    fate = finish_step<kAdjoint, kSpectral>(p, ph, sd, h, detail, tl);
-                    if (kStats) cnt.cyc[kCycFinish] += (unsigned long long)(clock64() - cf);
-                }
+            // the next step's draws and its flight: clear of every triangle
+            // by the table, or a query
+            const StepDraw sd = begin_step<kSpectral>(p, ph);
+            const float d = fminf(sd.d_abs, sd.d_ray);
+            uint32_t word = LXO_NO_HIT;
+            float3 sh = f3(0.0f, 0.0f, 0.0f);
+            uint32_t units;
+            const uint32_t clusters = cluster_mask(p.sc, ph.pos, ph.dir, d);
+            const bool clear = clear_flight(p.sc, ph.pos, ph.dir, d, units);
+            if (clear && clusters == 0u) {
+                to = kBulk;
+                if (kStats) step_histogram(p, ph.medium, 0, 0);
             } else {
-                fate = photon_step<kStats, kAdjoint, kSpectral>(p, ph, detail, cnt, tl);
+                to = clusters ? kReadyLayer : kReady;
+                const float ax = fabsf(ph.dir.x), ay = fabsf(ph.dir.y), az = fabsf(ph.dir.z);
+                const int k = (ax >= ay) ? ((ax >= az) ? 0 : 2) : ((ay >= az) ? 1 : 2);
+                const float dkz = pick(k, ph.dir.x, ph.dir.y, ph.dir.z);
+                sh.x = __fdiv_rn(pick(k, ph.dir.y, ph.dir.z, ph.dir.x), dkz);
+                sh.y = __fdiv_rn(pick(k, ph.dir.z, ph.dir.x, ph.dir.y), dkz);
+                sh.z = __fdiv_rn(1.0f, dkz);
+                word = (uint32_t)k | (clusters << 2) | (units << 16);
             }
-            if (stepped) {
-                ph.step++;
-                if (kStats) my_steps++;
-                if (fate < 0 && ph.step >= p.max_steps) {
-                    fate = LXO_FATE_TRUNCATED;
-                    detail = -1;
-                }
-                if (fate >= 0) {
-                    alive = false;
-                    pending = true;
-                }
-            }
+            const uint32_t ab = sd.d_abs <= sd.d_ray ? 0x80000000u : 0u;
+            q[0] = make_float4(ph.pos.x, ph.pos.y, ph.pos.z, __uint_as_float(__float_as_uint(d) | ab));
+            q[1] = make_float4(ph.dir.x, ph.dir.y, ph.dir.z, __uint_as_float(word));
+            q[4] = make_float4(sh.x, sh.y, sh.z, ph.wl);
+        } else if (fate >= 0) {
+            to = kFree;
+            q[0] = make_float4(ph.pos.x, ph.pos.y, ph.pos.z, __int_as_float(detail));
+            q[1] = make_float4(ph.dir.x, ph.dir.y, ph.dir.z, __int_as_float(fate));
         }
-        if (kStats) loop_cycles += (unsigned long long)(clock64() - c0);
+        if (to >= 0) {
+            q[2] = make_float4(ph.pol.x, ph.pol.y, ph.pol.z, ph.time);
+            q[3] = make_float4(__uint_as_float((uint32_t)ph.pid), __uint_as_float((uint32_t)(ph.pid >> 32)),
+                               __uint_as_float(ph.step),
+                               __uint_as_float(((uint32_t)ph.medium << 28) | (ph.last & kNoTri)));
+        }
+        __threadfence_block();
+        if (to >= 0) put(s_set[to], s);
+        __syncwarp();
+        lap(cnt.cyc[kCycDraw], got);
     }
     __syncthreads();
     for (int i = threadIdx.x; i < p.n_fates; i += blockDim.x)
         if (s_f[i]) atomicAdd(&p.out.fates[i], s_f[i]);
     if (kStats) {
-        atomicAdd(&p.out.stats[0], (unsigned long long)my_steps);
-        atomicAdd(&p.out.stats[1], (unsigned long long)cnt.nodes);
-        atomicAdd(&p.out.stats[2], (unsigned long long)cnt.leaves);
-        atomicAdd(&p.out.stats[3], (unsigned long long)cnt.tris);
-        atomicAdd(&p.out.stats[4], (unsigned long long)cnt.node_iters);
-        atomicAdd(&p.out.stats[5], (unsigned long long)cnt.leaf_iters);
-        atomicAdd(&p.out.stats[6], (unsigned long long)outer_iters);
-        atomicAdd(&p.out.stats[7], cnt.trav_cycles);
-        atomicAdd(&p.out.stats[8], loop_cycles);
-        for (int k = 0; k < kCycPhases; ++k) atomicAdd(&p.out.stats[29 + k], cnt.cyc[k]);
+        unsigned long long* o = p.out.stats;
+        atomicAdd(&o[0], (unsigned long long)cnt.steps);
+        atomicAdd(&o[1], (unsigned long long)cnt.nodes);
+        atomicAdd(&o[2], (unsigned long long)cnt.leaves);
+        atomicAdd(&o[3], (unsigned long long)cnt.tris);
+        atomicAdd(&o[4], (unsigned long long)cnt.node_iters);
+        atomicAdd(&o[5], (unsigned long long)cnt.leaf_iters);
+        atomicAdd(&o[6], (unsigned long long)cnt.batches);
+        atomicAdd(&o[7], cnt.cyc[kCycNode] + cnt.cyc[kCycLeaf] + cnt.cyc[kCycBegin]);
+        atomicAdd(&o[8], cnt.loop_cycles);
+        for (int k = 0; k < kCycPhases; ++k) atomicAdd(&o[29 + k], cnt.cyc[k]);
+        atomicAdd(&o[35], (unsigned long long)cnt.entries);
+        atomicAdd(&o[36], cnt.idle_cycles);
+        atomicAdd(&o[37], (unsigned long long)cnt.walks);
+        atomicAdd(&o[38], (unsigned long long)cnt.walk_iters);
     }
 }
 
@@ -1296,52 +1544,42 @@ cudaError_t launch_sample_source(const PropParams& p, float* pos, float* dir, fl
     return cudaGetLastError();
 }
 
-template <int kThreads, int kBudget>
-static cudaError_t launch_propagate_t(const PropParams& p, int sms, cudaStream_t st)
+cudaError_t launch_propagate(const PropParams& params, int device, cudaStream_t st)
 {
+    if (params.n == 0) return cudaSuccess;
+    PropParams p = params;
     const bool stats = (p.flags & LXO_FLAG_STATS) != 0;
     const bool adj = (p.flags & LXO_FLAG_ADJOINT) != 0;
-    auto kern = p.spectral ? (adj ? k_propagate<false, true, true, kThreads, kBudget>
-                                  : k_propagate<false, false, true, kThreads, kBudget>)
-                           : (adj ? k_propagate<false, true, false, kThreads, kBudget>
-                                  : k_propagate<false, false, false, kThreads, kBudget>);
-    if (stats)  // the counting build exists for the default shape only
-        kern = p.spectral ? (adj ? k_propagate<true, true, true, 256, kBudgetFull>
-                                 : k_propagate<true, false, true, 256, kBudgetFull>)
-                          : (adj ? k_propagate<true, true, false, 256, kBudgetFull>
-                                 : k_propagate<true, false, false, 256, kBudgetFull>);
-    const int threads = stats ? 256 : kThreads;
-    int per_sm = 0;
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, 0);
-    if (e != cudaSuccess) return e;
-    if (p.blocks_per_sm > 0 && (int)p.blocks_per_sm < per_sm) per_sm = (int)p.blocks_per_sm;
-    uint64_t blocks = (uint64_t)sms * (uint64_t)(per_sm > 0 ? per_sm : 1);
-    const uint64_t need = (p.n + threads - 1) / threads;
-    if (need < blocks) blocks = need;
-    kern<<<(unsigned)blocks, threads, 0, st>>>(p);
-    return cudaGetLastError();
-}
-
-// The register budget: the wide one (48 registers) when the launch asks for
-// at most kBudgetWide CTAs of 256 threads per SM, or by default for the
-// adjoint build; else the full-occupancy one (32 registers).
-template <int kThreads>
-static cudaError_t launch_propagate_b(const PropParams& p, int sms, cudaStream_t st)
-{
-    const int per256 = 256 / kThreads;
-    const bool adj = (p.flags & LXO_FLAG_ADJOINT) != 0;
-    const bool wide = p.blocks_per_sm ? (int)p.blocks_per_sm <= kBudgetWide * per256 : adj;
-    return wide ? launch_propagate_t<kThreads, kBudgetWide>(p, sms, st)
-                : launch_propagate_t<kThreads, kBudgetFull>(p, sms, st);
-}
-
-cudaError_t launch_propagate(const PropParams& p, int device, cudaStream_t st)
-{
-    if (p.n == 0) return cudaSuccess;
+    auto kern = p.spectral ? (adj ? k_propagate<false, true, true> : k_propagate<false, false, true>)
+                           : (adj ? k_propagate<false, true, false> : k_propagate<false, false, false>);
+    if (stats)
+        kern = p.spectral ? (adj ? k_propagate<true, true, true> : k_propagate<true, false, true>)
+                          : (adj ? k_propagate<true, true, false> : k_propagate<true, false, false>);
     int sms = 0;
     cudaError_t e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
     if (e != cudaSuccess) return e;
-    return p.block_threads == 128 ? launch_propagate_b<128>(p, sms, st) : launch_propagate_b<256>(p, sms, st);
+    // slots per CTA: what kPoolCtas CTAs leave of the SM's shared memory (164
+    // KiB of it for the forward builds, all of it with the adjoint tallies)
+    cudaFuncAttributes fa;
+    e = cudaFuncGetAttributes(&fa, kern);
+    if (e != cudaSuccess) return e;
+    p.tally_stride = adj ? (p.adj_k | 1) : 0;
+    const size_t per_slot = sizeof(float4) * kSlotF4 + sizeof(float) * p.tally_stride;
+    const size_t room = (size_t)(adj ? 227 : LXO_POOL_KB) * 1024 / kPoolCtas - 1024 - fa.sharedSizeBytes;
+    const uint64_t slots = std::min<uint64_t>(kMaxSlots, room / per_slot / 32 * 32);
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(slots * per_slot));
+    if (e != cudaSuccess) return e;
+    int per_sm = 0;
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kPoolThreads, slots * per_slot);
+    if (e != cudaSuccess) return e;
+    // a launch shape set by the caller limits the threads per SM
+    if (p.blocks_per_sm > 0)
+        per_sm = std::min(per_sm, (int)((p.blocks_per_sm * p.block_threads + kPoolThreads - 1) / kPoolThreads));
+    per_sm = std::max(1, per_sm);
+    uint64_t blocks = std::min<uint64_t>((uint64_t)sms * per_sm, p.n);
+    p.slots = (int)std::min<uint64_t>(slots, (p.n + blocks - 1) / blocks);
+    kern<<<(unsigned)blocks, kPoolThreads, slots * per_slot, st>>>(p);
+    return cudaGetLastError();
 }
 
 // ---------------------------------------------------------------------------
