@@ -47,16 +47,13 @@ struct U4 {
     float u0, u1, u2, u3;
 };
 
-#ifndef LXO_PHILOX_UNROLL
-#define LXO_PHILOX_UNROLL 10
-#endif
-#ifndef LXO_PHILOX_INLINE
-#define LXO_PHILOX_INLINE __forceinline__
-#endif
-constexpr int kPhiloxUnroll = LXO_PHILOX_UNROLL;
-static __device__ LXO_PHILOX_INLINE uint4 philox4x32_10(uint4 c, uint2 k)
+// kRounds: rounds per iteration of the code (10: no loop; 1: a tenth of the
+// code, for the places that are not hot -- instruction fetch is what bounds
+// the photon loop)
+template <int kRounds = 10>
+__device__ __forceinline__ uint4 philox4x32_10(uint4 c, uint2 k)
 {
-#pragma unroll kPhiloxUnroll
+#pragma unroll kRounds
     for (int r = 0; r < 10; ++r) {
         uint32_t hi0 = __umulhi(0xD2511F53u, c.x), lo0 = 0xD2511F53u * c.x;
         uint32_t hi1 = __umulhi(0xCD9E8D57u, c.z), lo1 = 0xCD9E8D57u * c.z;
@@ -73,9 +70,10 @@ __device__ __forceinline__ float u01(uint32_t x)
     return __fmul_rn(__uint2float_rn(x >> 9) + 0.5f, 1.1920928955078125e-07f);
 }
 
+template <int kRounds = 10>
 __device__ __forceinline__ U4 draw4(uint64_t seed, uint64_t pid, uint32_t step, uint32_t draw)
 {
-    uint4 o = philox4x32_10(make_uint4((uint32_t)pid, (uint32_t)(pid >> 32), step, draw),
+    uint4 o = philox4x32_10<kRounds>(make_uint4((uint32_t)pid, (uint32_t)(pid >> 32), step, draw),
                             make_uint2((uint32_t)seed, (uint32_t)(seed >> 32)));
     return U4{u01(o.x), u01(o.y), u01(o.z), u01(o.w)};
 }
@@ -110,36 +108,29 @@ __device__ __forceinline__ void onb(float3 n, float3& t1, float3& t2)
 struct WRay {
     float ox, oy, oz;
     float Sx, Sy, Sz;
-    int kx, ky, kz;
+    int kz;   // axis of the direction's largest component
 };
 
 __device__ __forceinline__ float pick(int k, float x, float y, float z) { return k == 0 ? x : (k == 1 ? y : z); }
 
+// The axes kx, ky are not swapped for a negative component along kz: the swap
+// negates U, V, W, det and T exactly, so every hit and t is the same.
+__device__ __forceinline__ int shear(float3 d, float3& S)
+{
+    const float ax = fabsf(d.x), ay = fabsf(d.y), az = fabsf(d.z);
+    const int kz = (ax >= ay) ? ((ax >= az) ? 0 : 2) : ((ay >= az) ? 1 : 2);
+    const float dkz = pick(kz, d.x, d.y, d.z);
+    S.x = __fdiv_rn(pick(kz, d.y, d.z, d.x), dkz);
+    S.y = __fdiv_rn(pick(kz, d.z, d.x, d.y), dkz);
+    S.z = __fdiv_rn(1.0f, dkz);
+    return kz;
+}
+
 __device__ __forceinline__ WRay wray_setup(float3 o, float3 d)
 {
-    WRay r;
-    float ax = fabsf(d.x), ay = fabsf(d.y), az = fabsf(d.z);
-    int kz = (ax >= ay) ? ((ax >= az) ? 0 : 2) : ((ay >= az) ? 1 : 2);
-    int kx = kz + 1;
-    if (kx == 3) kx = 0;
-    int ky = kx + 1;
-    if (ky == 3) ky = 0;
-    float dkz = pick(kz, d.x, d.y, d.z);
-    if (dkz < 0.0f) {
-        int t = kx;
-        kx = ky;
-        ky = t;
-    }
-    r.kx = kx;
-    r.ky = ky;
-    r.kz = kz;
-    r.Sx = __fdiv_rn(pick(kx, d.x, d.y, d.z), dkz);
-    r.Sy = __fdiv_rn(pick(ky, d.x, d.y, d.z), dkz);
-    r.Sz = __fdiv_rn(1.0f, dkz);
-    r.ox = o.x;
-    r.oy = o.y;
-    r.oz = o.z;
-    return r;
+    float3 S;
+    const int kz = shear(d, S);
+    return WRay{o.x, o.y, o.z, S.x, S.y, S.z, kz};
 }
 
 // The edge functions again in double, for when one of them rounded to zero
@@ -159,18 +150,20 @@ __device__ __forceinline__ bool wray_hit(const WRay& r, float4 a, float4 b, floa
     const float A0 = __fsub_rn(a.x, r.ox), A1 = __fsub_rn(a.y, r.oy), A2 = __fsub_rn(a.z, r.oz);
     const float B0 = __fsub_rn(a.w, r.ox), B1 = __fsub_rn(b.x, r.oy), B2 = __fsub_rn(b.y, r.oz);
     const float C0 = __fsub_rn(b.z, r.ox), C1 = __fsub_rn(b.w, r.oy), C2 = __fsub_rn(c.x, r.oz);
-    const float Akz = pick(r.kz, A0, A1, A2), Bkz = pick(r.kz, B0, B1, B2), Ckz = pick(r.kz, C0, C1, C2);
-    const float Ax = __fsub_rn(pick(r.kx, A0, A1, A2), __fmul_rn(r.Sx, Akz));
-    const float Ay = __fsub_rn(pick(r.ky, A0, A1, A2), __fmul_rn(r.Sy, Akz));
-    const float Bx = __fsub_rn(pick(r.kx, B0, B1, B2), __fmul_rn(r.Sx, Bkz));
-    const float By = __fsub_rn(pick(r.ky, B0, B1, B2), __fmul_rn(r.Sy, Bkz));
-    const float Cx = __fsub_rn(pick(r.kx, C0, C1, C2), __fmul_rn(r.Sx, Ckz));
-    const float Cy = __fsub_rn(pick(r.ky, C0, C1, C2), __fmul_rn(r.Sy, Ckz));
+    // axes kx, ky = the two after kz in turn
+    const bool k0 = r.kz == 0, k1 = r.kz == 1;
+    const float Akz = k0 ? A0 : (k1 ? A1 : A2), Bkz = k0 ? B0 : (k1 ? B1 : B2), Ckz = k0 ? C0 : (k1 ? C1 : C2);
+    const float Ax = __fsub_rn(k0 ? A1 : (k1 ? A2 : A0), __fmul_rn(r.Sx, Akz));
+    const float Ay = __fsub_rn(k0 ? A2 : (k1 ? A0 : A1), __fmul_rn(r.Sy, Akz));
+    const float Bx = __fsub_rn(k0 ? B1 : (k1 ? B2 : B0), __fmul_rn(r.Sx, Bkz));
+    const float By = __fsub_rn(k0 ? B2 : (k1 ? B0 : B1), __fmul_rn(r.Sy, Bkz));
+    const float Cx = __fsub_rn(k0 ? C1 : (k1 ? C2 : C0), __fmul_rn(r.Sx, Ckz));
+    const float Cy = __fsub_rn(k0 ? C2 : (k1 ? C0 : C1), __fmul_rn(r.Sy, Ckz));
     float U = __fsub_rn(__fmul_rn(Cx, By), __fmul_rn(Cy, Bx));
     float V = __fsub_rn(__fmul_rn(Ax, Cy), __fmul_rn(Ay, Cx));
     float W = __fsub_rn(__fmul_rn(Bx, Ay), __fmul_rn(By, Ax));
-    if (U == 0.0f || V == 0.0f || W == 0.0f) edges_fp64(Ax, Ay, Bx, By, Cx, Cy, U, V, W);
-    if ((U < 0.0f || V < 0.0f || W < 0.0f) && (U > 0.0f || V > 0.0f || W > 0.0f)) return false;
+    if (fminf(fminf(fabsf(U), fabsf(V)), fabsf(W)) == 0.0f) edges_fp64(Ax, Ay, Bx, By, Cx, Cy, U, V, W);
+    if (fminf(fminf(U, V), W) < 0.0f && fmaxf(fmaxf(U, V), W) > 0.0f) return false;
     const float det = __fadd_rn(__fadd_rn(U, V), W);
     if (det == 0.0f) return false;
     const float Az = __fmul_rn(r.Sz, Akz), Bz = __fmul_rn(r.Sz, Bkz), Cz = __fmul_rn(r.Sz, Ckz);
@@ -248,8 +241,6 @@ __device__ __forceinline__ void test_leaf(const Scene& sc, const WRay& wr, int r
 // from the query's slot, the closest triangle known by its record.  One
 // triangle a call, since the lanes of a warp hold leaves of different sizes
 // (all of a leaf at once ran 4.4 tests a call for 1.5 triangles a leaf).
-// The axes are not swapped for a negative dkz: the swap negates U, V, W, det
-// and T exactly, so every hit and t stays the same.
 __device__ __forceinline__ void slot_triangle(const Scene& sc, const float4* q, int kz, uint32_t skip, int& leaf,
                                               float& bt, uint32_t& best_rec, int* bounds_err)
 {
@@ -263,8 +254,7 @@ __device__ __forceinline__ void slot_triangle(const Scene& sc, const float4* q, 
     const float4* tr = sc.tris + 3 * (size_t)r;
     const float4 a = __ldg(tr + 0), b = __ldg(tr + 1), c = __ldg(tr + 2);
     const float4 o = q[0], sh = q[4];
-    const int kx = kz == 2 ? 0 : kz + 1, ky = kz == 0 ? 2 : kz - 1;
-    const WRay wr{o.x, o.y, o.z, sh.x, sh.y, sh.z, kx, ky, kz};
+    const WRay wr{o.x, o.y, o.z, sh.x, sh.y, sh.z, kz};
     const uint32_t id = __float_as_uint(c.y);
     float t;
     if (id != skip && wray_hit(wr, a, b, c, bt, t)) {
@@ -332,7 +322,9 @@ __device__ __forceinline__ void enter_clusters(const Scene& sc, uint32_t mask, f
             const float fj1 = fminf(floorf((fmaxf(v1, v2) + cl.delta - cl.v0) * cl.inv_cell), (float)(cl.nv - 1));
             if (!(fi0 <= fi1) || !(fj0 <= fj1)) continue;  // outside the cluster's grid
             if ((fi1 - fi0 + 1.0f) * (fj1 - fj0 + 1.0f) <= (float)kMaxCellsPerRay) {
+#pragma unroll 1
                 for (int j = (int)fj0; j <= (int)fj1; ++j)
+#pragma unroll 1
                     for (int i = (int)fi0; i <= (int)fi1; ++i) {
                         if (LXO_CHECK_BOUNDS && (i < 0 || j < 0 || i >= cl.nu || j >= cl.nv)) continue;
                         const int r = __ldg(&cl.cells[(size_t)j * cl.nu + i]);
@@ -520,7 +512,7 @@ __device__ __forceinline__ bool inside_poly(const SourceDev& s, float x, float y
 __device__ __forceinline__ float emission_delay(const PropParams& p, uint64_t pid, const TimeProfile& tp)
 {
     if (tp.tau_s == 0.0f && tp.tau_t == 0.0f) return 0.0f;
-    const U4 u = draw4(p.seed, pid, kSourceStep, 0xFFFFFFFFu);
+    const U4 u = draw4<1>(p.seed, pid, kSourceStep, 0xFFFFFFFFu);
     const float tau = u.u0 < tp.f_s ? tp.tau_s : tp.tau_t;
     return -tau * logf(u.u1);
 }
@@ -530,7 +522,7 @@ __device__ __forceinline__ float emission_delay(const PropParams& p, uint64_t pi
 __device__ __forceinline__ float emission_wavelength(const PropParams& p, uint64_t pid, const Spectrum& sp)
 {
     if (sp.sigma == 0.0f) return sp.mean;
-    const U4 u = draw4(p.seed, pid, kSourceStep, 0xFFFFFFFFu);
+    const U4 u = draw4<1>(p.seed, pid, kSourceStep, 0xFFFFFFFFu);
     float s, c;
     sincospif(2.0f * u.u3, &s, &c);
     return fmaf(sp.sigma, sqrtf(-2.0f * logf(u.u2)) * c, sp.mean);
@@ -566,7 +558,7 @@ __device__ Photon make_event_photon(const PropParams& p, uint64_t idx)
     ph.wl = p.spectral ? emission_wavelength(p, ph.pid, ev.spec) : 0.0f;
     ph.last = LXO_NO_HIT;
     ph.step = 0;
-    const U4 u = draw4(p.seed, ph.pid, kSourceStep, 0);
+    const U4 u = draw4<1>(p.seed, ph.pid, kSourceStep, 0);
     const float c = 2.0f * u.u0 - 1.0f, sn = sqrtf(fmaxf(0.0f, 1.0f - c * c));
     float sp, cp;
     sincospif(2.0f * u.u1, &sp, &cp);
@@ -580,7 +572,7 @@ __device__ Photon make_event_photon(const PropParams& p, uint64_t idx)
         if (ev.kind == LXO_SRC_BALL) {
 #pragma unroll 1
             for (int tr = 0; tr < kMaxTries; ++tr) {
-                const U4 w = draw4(p.seed, ph.pid, kSourceStep, 1 + tr);
+                const U4 w = draw4<1>(p.seed, ph.pid, kSourceStep, 1 + tr);
                 const float x = ev.radius * (2.0f * w.u0 - 1.0f), y = ev.radius * (2.0f * w.u1 - 1.0f),
                             z = ev.radius * (2.0f * w.u2 - 1.0f);
                 if (x * x + y * y + z * z <= ev.radius * ev.radius) {
@@ -593,10 +585,7 @@ __device__ Photon make_event_photon(const PropParams& p, uint64_t idx)
     return ph;
 }
 
-#ifndef LXO_MAKE_INLINE
-#define LXO_MAKE_INLINE
-#endif
-__device__ LXO_MAKE_INLINE Photon make_photon(const PropParams& p, uint64_t idx)
+__device__ Photon make_photon(const PropParams& p, uint64_t idx)
 {
     if (p.n_events) return make_event_photon(p, idx);
     const SourceDev& s = p.src;
@@ -614,7 +603,7 @@ __device__ LXO_MAKE_INLINE Photon make_photon(const PropParams& p, uint64_t idx)
         ph.pol = normalize(e - dot(e, ph.dir) * ph.dir);
         return ph;
     }
-    const U4 u = draw4(p.seed, ph.pid, kSourceStep, 0);
+    const U4 u = draw4<1>(p.seed, ph.pid, kSourceStep, 0);
     const float c = 2.0f * u.u0 - 1.0f, sn = sqrtf(fmaxf(0.0f, 1.0f - c * c));
     float sp, cp;
     sincospif(2.0f * u.u1, &sp, &cp);
@@ -629,7 +618,7 @@ __device__ LXO_MAKE_INLINE Photon make_photon(const PropParams& p, uint64_t idx)
         ph.pos = f3(s.center[0], s.center[1], s.center[2]);
 #pragma unroll 1
         for (int tr = 0; tr < kMaxTries; ++tr) {
-            const U4 w = draw4(p.seed, ph.pid, kSourceStep, 1 + tr);
+            const U4 w = draw4<1>(p.seed, ph.pid, kSourceStep, 1 + tr);
             const float x = s.radius * (2.0f * w.u0 - 1.0f), y = s.radius * (2.0f * w.u1 - 1.0f),
                         z = s.radius * (2.0f * w.u2 - 1.0f);
             if (x * x + y * y + z * z <= s.radius * s.radius) {
@@ -641,7 +630,7 @@ __device__ LXO_MAKE_INLINE Photon make_photon(const PropParams& p, uint64_t idx)
         ph.pos = f3(0.0f, 0.0f, s.z_min + u.u3 * (s.z_max - s.z_min));
 #pragma unroll 1
         for (int tr = 0; tr < kMaxTries; ++tr) {
-            const U4 w = draw4(p.seed, ph.pid, kSourceStep, 1 + tr);
+            const U4 w = draw4<1>(p.seed, ph.pid, kSourceStep, 1 + tr);
             float r = s.radius * sqrtf(w.u0), sa, ca;
             sincospif(2.0f * w.u1, &sa, &ca);
             if (inside_poly(s, r * ca, r * sa, w.u1)) {
@@ -864,7 +853,7 @@ __device__ __forceinline__ int surface_event(const PropParams& p, Photon& ph, fl
     const uint32_t id = __float_as_uint(vc.y);
     const uint2 at = make_uint2(__float_as_uint(vc.z), __float_as_uint(vc.w));
     // the step's first draw again (its first two uniforms gave the distances)
-    const U4 u = draw4(p.seed, ph.pid, ph.step, 0);
+    const U4 u = draw4<1>(p.seed, ph.pid, ph.step, 0);
     const float3 e1 = f3(va.w - va.x, vb.x - va.y, vb.y - va.z);
     const float3 e2 = f3(vb.z - va.x, vb.w - va.y, vc.x - va.z);
     const float3 ng = normalize(cross(e1, e2));
@@ -926,7 +915,7 @@ __device__ __forceinline__ int surface_event(const PropParams& p, Photon& ph, fl
             return LXO_FATE_SURF_ABS;
         }
         if (kAdjoint && ss >= 0) tl[base_k + 1] += 1.0f;
-        specular = draw4(p.seed, ph.pid, ph.step, 1).u3 < sf.wspec;
+        specular = draw4<1>(p.seed, ph.pid, ph.step, 1).u3 < sf.wspec;
     } else {
         detail = (int)id;
         return LXO_FATE_GEOM_ERR;
@@ -957,12 +946,19 @@ __device__ __forceinline__ int surface_event(const PropParams& p, Photon& ph, fl
 // Flights that meet nothing need no query: the walk grid's empty cubes clear
 // them (over half of the DARWIN-scale mesh's steps), which pays only because
 // the lanes of the others are then filled with other photons.
+// Instruction fetch is what is left: the requests that miss the SM's
+// instruction cache came at the same 0.515 per cycle and GPC in three versions
+// of this loop, so hot code is kept short (82 KB -> 75 KB: 8 to 12 % less
+// time).
+// Launch shape: CTAs of kPoolThreads threads, kPoolCtas per SM: 18 warps of 56
+// registers each; 2e7 photons on the DARWIN-scale mesh / 3e6 on the 50 cm TPC
+// took 63.1 / 11.4 ms, with 2 x 640 threads of 48 registers 66.5 / 12.0, with
+// 2 x 512 of 64 66.8 / 11.4, with 3 x 384 of 56 66.4 / 11.4.
 // Measured (1e8 photons on the DARWIN-scale mesh / 3e6 on the 50 cm TPC with
 // dispersion / 2e6 on the mesh without electrodes, GB300): 503 / 21.0 / 17.7
-// ms before, 359 / 13.5 / 12.2 ms now.
-// Launch shape: CTAs of kPoolThreads threads, kPoolCtas per SM.
+// ms for the loop before, 316 / 12.0 / 10.5 ms now.
 #ifndef LXO_POOL_THREADS
-#define LXO_POOL_THREADS 640
+#define LXO_POOL_THREADS 576
 #endif
 #ifndef LXO_POOL_CTAS
 #define LXO_POOL_CTAS 2
@@ -1165,15 +1161,15 @@ __device__ __forceinline__ uint32_t cluster_mask(const Scene& sc, float3 o, floa
     const float t = tmax * kBoxSlack;
     const float ex = fmaf(t, d.x, o.x), ey = fmaf(t, d.y, o.y), ez = fmaf(t, d.z, o.z);
     // (fminf and fmaxf skip the NaN of an unlimited ray with d = 0 along the axis)
-    const float l[3] = {fminf(o.x, ex), fminf(o.y, ey), fminf(o.z, ez)};
-    const float h[3] = {fmaxf(o.x, ex), fmaxf(o.y, ey), fmaxf(o.z, ez)};
     uint32_t m = 0;
-#pragma unroll
+#pragma unroll 1
     for (int a = 0; a < 3; ++a) {
         if (!((sc.layer_axes >> a) & 1u)) continue;
+        const float b = pick(a, o.x, o.y, o.z), e = pick(a, ex, ey, ez);
+        const float l = fminf(b, e), h = fmaxf(b, e);
 #pragma unroll
         for (int c = 0; c < kMaxClusters; ++c)   // unused entries are empty slabs
-            m |= h[a] >= sc.layer_lo[a][c] && l[a] <= sc.layer_hi[a][c] ? 1u << c : 0u;
+            m |= h >= sc.layer_lo[a][c] && l <= sc.layer_hi[a][c] ? 1u << c : 0u;
     }
     return m;
 }
@@ -1472,12 +1468,7 @@ __global__ void __launch_bounds__(kPoolThreads, kPoolCtas) k_propagate(const __g
                 if (kStats) step_histogram(p, ph.medium, 0, 0);
             } else {
                 to = clusters ? kReadyLayer : kReady;
-                const float ax = fabsf(ph.dir.x), ay = fabsf(ph.dir.y), az = fabsf(ph.dir.z);
-                const int k = (ax >= ay) ? ((ax >= az) ? 0 : 2) : ((ay >= az) ? 1 : 2);
-                const float dkz = pick(k, ph.dir.x, ph.dir.y, ph.dir.z);
-                sh.x = __fdiv_rn(pick(k, ph.dir.y, ph.dir.z, ph.dir.x), dkz);
-                sh.y = __fdiv_rn(pick(k, ph.dir.z, ph.dir.x, ph.dir.y), dkz);
-                sh.z = __fdiv_rn(1.0f, dkz);
+                const int k = shear(ph.dir, sh);
                 word = (uint32_t)k | (clusters << 2) | (units << 16);
             }
             const uint32_t ab = sd.d_abs <= sd.d_ray ? 0x80000000u : 0u;
