@@ -175,16 +175,11 @@ __device__ __forceinline__ bool wray_hit(const WRay& r, float4 a, float4 b, floa
 }
 
 // ---------------------------------------------------------------------------
-// BVH traversal: closest hit with t in (0, tmax], skipping one triangle,
-// ties to the smallest triangle id.
+// Closest hit with t in (0, tmax], skipping one triangle, ties to the smallest
+// triangle id: layers entered by their cells, the rest of the scene walked
+// through the grid (or searched by its main tree).
 // ---------------------------------------------------------------------------
 constexpr float kBoxSlack = 1.0f + 1.0f / 65536.0f;
-
-struct Hit {
-    uint32_t id;   // triangle id (LXO_NO_HIT on miss)
-    uint32_t rec;  // record index in leaf order
-    float t;
-};
 
 // The reciprocal without IEEE rounding (1 ulp): the slab test is conservative
 // by the boxes' margin and the slack, so the hits are the same.
@@ -194,6 +189,9 @@ __device__ __forceinline__ float fast_inv(float d)
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(fabsf(d) < 1e-20f ? 1e-20f : d));
     return r;
 }
+
+constexpr int kSlotF4 = 5;            // float4 per query slot in shared memory (see load_slot)
+constexpr uint32_t kNoTri = 0x0FFFFFFFu;  // "no triangle" in 28 bits (ids stay below 2^28 - 1)
 
 // Counting build: what one lane counts (warp-wide figures by lane 0).  Lane
 // cycles by phase of the photon loop, a warp's clock times the lanes at work:
@@ -209,40 +207,12 @@ struct Counters {
     unsigned long long cyc[kCycPhases];
 };
 
-// Leaf test of one leaf reference: every triangle of the leaf through the
-// exact watertight test, keeping (t, id) minimal in that order.
-__device__ __forceinline__ void test_leaf(const Scene& sc, const WRay& wr, int ref, uint32_t skip, float& bt,
-                                          uint32_t& best, uint32_t& best_rec, int* bounds_err)
-{
-    const uint32_t enc = ~(uint32_t)ref;
-    const uint32_t first = enc >> 3, count = (enc & 7u) + 1u;
-    if (LXO_CHECK_BOUNDS && (uint64_t)first + count > sc.n_records) {
-        atomicOr(bounds_err, kErrBounds);
-        return;
-    }
-    for (uint32_t k = 0; k < count; ++k) {
-        const float4* tr = sc.tris + 3 * (size_t)(first + k);
-        const float4 a = __ldg(tr + 0), b = __ldg(tr + 1), c = __ldg(tr + 2);
-        const uint32_t id = __float_as_uint(c.y);
-        if (id == skip) continue;
-        float t;
-        if (wray_hit(wr, a, b, c, bt, t)) {
-            if (t < bt || (t == bt && (best == LXO_NO_HIT || id < best))) {
-                bt = t;
-                best = id;
-                best_rec = first + k;
-            }
-        }
-    }
-}
-
-// The next triangle of a leaf for a query of the photon pool, the leaf
-// reference moved on past it (0 after the last): origin and shear constants
-// from the query's slot, the closest triangle known by its record.  One
-// triangle a call, since the lanes of a warp hold leaves of different sizes
-// (all of a leaf at once ran 4.4 tests a call for 1.5 triangles a leaf).
-__device__ __forceinline__ void slot_triangle(const Scene& sc, const float4* q, int kz, uint32_t skip, int& leaf,
-                                              float& bt, uint32_t& best_rec, int* bounds_err)
+// The next triangle of a leaf, the leaf reference moved on past it (0 after the
+// last); the closest triangle known by its record.  One triangle a call, since
+// the lanes of a warp hold leaves of different sizes (all of a leaf at once
+// ran 4.4 tests a call for 1.5 triangles a leaf).
+__device__ __forceinline__ void triangle(const Scene& sc, const WRay& wr, uint32_t skip, int& leaf, float& bt,
+                                         uint32_t& best_rec, int* bounds_err)
 {
     const uint32_t enc = ~(uint32_t)leaf;
     const uint32_t r = enc >> 3;
@@ -253,8 +223,6 @@ __device__ __forceinline__ void slot_triangle(const Scene& sc, const float4* q, 
     }
     const float4* tr = sc.tris + 3 * (size_t)r;
     const float4 a = __ldg(tr + 0), b = __ldg(tr + 1), c = __ldg(tr + 2);
-    const float4 o = q[0], sh = q[4];
-    const WRay wr{o.x, o.y, o.z, sh.x, sh.y, sh.z, kz};
     const uint32_t id = __float_as_uint(c.y);
     float t;
     if (id != skip && wray_hit(wr, a, b, c, bt, t)) {
@@ -271,32 +239,6 @@ constexpr int kDone = INT32_MIN + 1;  // bottom of the stack
 constexpr int kWalk = INT32_MIN + 2;  // back to the walk through the grid
 
 __device__ __forceinline__ bool is_leaf(int node) { return (uint32_t)node > (uint32_t)kWalk; }
-
-// Traversal state of one ray (its stack lives in a separate local
-// array of kStackSize entries).
-struct TravState {
-    WRay wr;
-    float ix, iy, iz, oix, oiy, oiz;
-    uint32_t skip;
-    float bt;
-    uint32_t best, best_rec;
-    int node, leaf, sp;
-};
-
-// The per-ray constants of a query of ray (o, d) skipping triangle `skip`:
-// the watertight test's shear and the slab test's inverse direction.
-__device__ __forceinline__ void trav_setup(const Scene& sc, float3 o, float3 d, uint32_t skip,
-                                           TravState& ts)
-{
-    ts.wr = wray_setup(o, d);
-    ts.ix = fast_inv(d.x) * sc.grid_h;
-    ts.iy = fast_inv(d.y) * sc.grid_h;
-    ts.iz = fast_inv(d.z) * sc.grid_h;
-    ts.oix = fmaf(o.x, sc.grid_inv, sc.grid_off[0]) * ts.ix;
-    ts.oiy = fmaf(o.y, sc.grid_inv, sc.grid_off[1]) * ts.iy;
-    ts.oiz = fmaf(o.z, sc.grid_inv, sc.grid_off[2]) * ts.iz;
-    ts.skip = skip;
-}
 
 // Pushes the entries of the planar clusters in `mask` for a ray with t in
 // (0, tmax]: a ray crossing the slab within a few grid cells starts at those
@@ -337,32 +279,51 @@ __device__ __forceinline__ void enter_clusters(const Scene& sc, uint32_t mask, f
     }
 }
 
-// Enters the forest for a query with t in (0, tmax] (after trav_setup).
-__device__ __forceinline__ void trav_enter(const Scene& sc, float3 o, float3 d, float tmax, TravState& ts,
-                                           int* stack)
+// A ray for the slab test in grid space: i = 1 / direction, oi = origin * i.
+struct RayInv {
+    float ix, iy, iz, oix, oiy, oiz;
+};
+
+__device__ __forceinline__ RayInv ray_inv(const Scene& sc, float3 o, float3 d)
 {
-    ts.bt = tmax;
-    ts.best = LXO_NO_HIT;
-    ts.best_rec = 0;
-    stack[0] = kDone;
-    int sp = 1;
-    enter_clusters(sc, (1u << sc.n_clusters) - 1u, o, d, tmax, stack, sp);
-    ts.node = sc.main_root != kEmptyChild ? sc.main_root : stack[--sp];
-    ts.leaf = 0;  // parked leaf (0 = none: reference 0 is an internal node, never a leaf)
-    ts.sp = sp;
+    RayInv r;
+    r.ix = fast_inv(d.x) * sc.grid_h;
+    r.iy = fast_inv(d.y) * sc.grid_h;
+    r.iz = fast_inv(d.z) * sc.grid_h;
+    r.oix = fmaf(o.x, sc.grid_inv, sc.grid_off[0]) * r.ix;
+    r.oiy = fmaf(o.y, sc.grid_inv, sc.grid_off[1]) * r.iy;
+    r.oiz = fmaf(o.z, sc.grid_inv, sc.grid_off[2]) * r.iz;
+    return r;
 }
 
-__device__ __forceinline__ void trav_begin(const Scene& sc, float3 o, float3 d, uint32_t skip, float tmax,
-                                           TravState& ts, int* stack)
+// State of a query: next node (kDone: finished), stack entries, axis kz,
+// closest hit so far (t and record), and how far its walk has come.
+struct Query {
+    int node, sp, kz;
+    float bt, tw;
+    uint32_t rec;
+};
+
+// Starts a query with t in (0, tmax]: the layers in `clusters` wait on the
+// stack while the grid is walked from `clear` on (the main tree searched, if
+// that is negative: the ray starts outside the grid).
+__device__ __forceinline__ Query begin_query(const Scene& sc, float3 o, float3 d, int kz, float tmax, uint32_t clusters,
+                                             float clear, int* stack)
 {
-    trav_setup(sc, o, d, skip, ts);
-    trav_enter(sc, o, d, tmax, ts, stack);
+    Query c{kWalk, 1, kz, tmax, clear, LXO_NO_HIT};
+    stack[0] = kDone;
+    if (clusters) enter_clusters(sc, clusters, o, d, tmax, stack, c.sp);
+    if (!(clear >= 0.0f)) {
+        c.node = sc.main_root;
+        if (c.node == kEmptyChild) c.node = stack[--c.sp];
+    }
+    return c;
 }
 
 // One visit: the two children's boxes against the ray; descends into the
 // nearer child hit and pushes the other, or pops.
-__device__ __forceinline__ void node_visit(const Scene& sc, float ix, float iy, float iz, float oix, float oiy,
-                                           float oiz, float lim, int& node, int* stack, int& sp, int* err)
+__device__ __forceinline__ void node_visit(const Scene& sc, const RayInv& r, float lim, int& node, int* stack, int& sp,
+                                           int* err)
 {
     if (LXO_CHECK_BOUNDS && (uint32_t)node >= sc.n_nodes) {
         atomicOr(err, kErrBounds);
@@ -373,12 +334,12 @@ __device__ __forceinline__ void node_visit(const Scene& sc, float ix, float iy, 
     const float4* nd = sc.nodes + 4 * (size_t)node;
     const float4 nx = __ldg(nd + 0), ny = __ldg(nd + 1), nz = __ldg(nd + 2);
     const int4 cr = __ldg(reinterpret_cast<const int4*>(nd + 3));
-    const float ax0 = fmaf(nx.x, ix, -oix), ax1 = fmaf(nx.y, ix, -oix);
-    const float ay0 = fmaf(ny.x, iy, -oiy), ay1 = fmaf(ny.y, iy, -oiy);
-    const float az0 = fmaf(nz.x, iz, -oiz), az1 = fmaf(nz.y, iz, -oiz);
-    const float bx0 = fmaf(nx.z, ix, -oix), bx1 = fmaf(nx.w, ix, -oix);
-    const float by0 = fmaf(ny.z, iy, -oiy), by1 = fmaf(ny.w, iy, -oiy);
-    const float bz0 = fmaf(nz.z, iz, -oiz), bz1 = fmaf(nz.w, iz, -oiz);
+    const float ax0 = fmaf(nx.x, r.ix, -r.oix), ax1 = fmaf(nx.y, r.ix, -r.oix);
+    const float ay0 = fmaf(ny.x, r.iy, -r.oiy), ay1 = fmaf(ny.y, r.iy, -r.oiy);
+    const float az0 = fmaf(nz.x, r.iz, -r.oiz), az1 = fmaf(nz.y, r.iz, -r.oiz);
+    const float bx0 = fmaf(nx.z, r.ix, -r.oix), bx1 = fmaf(nx.w, r.ix, -r.oix);
+    const float by0 = fmaf(ny.z, r.iy, -r.oiy), by1 = fmaf(ny.w, r.iy, -r.oiy);
+    const float bz0 = fmaf(nz.z, r.iz, -r.oiz), bz1 = fmaf(nz.w, r.iz, -r.oiz);
     const float an = fmaxf(fmaxf(fminf(ax0, ax1), fminf(ay0, ay1)), fmaxf(fminf(az0, az1), 0.0f));
     const float af = fminf(fminf(fmaxf(ax0, ax1), fmaxf(ay0, ay1)), fminf(fmaxf(az0, az1), lim));
     const float bn = fmaxf(fmaxf(fminf(bx0, bx1), fminf(by0, by1)), fmaxf(fminf(bz0, bz1), 0.0f));
@@ -404,70 +365,330 @@ __device__ __forceinline__ void node_visit(const Scene& sc, float ix, float iy, 
     if (!(ha || hb)) node = stack[--sp];
 }
 
-// "While-while" traversal with postponed leaves (Aila & Laine, HPG 2009): a
-// lane that reaches a leaf parks it and keeps descending until every active
-// lane of the warp holds a leaf; then the warp tests leaves together.
-__device__ void trav_run(const Scene& sc, TravState& ts, int* stack, int* err)
+// Distance at which a ray leaves the cube of k cells (an octant's) that starts
+// with its cell (x, y, z): in grid space, i = 1 / direction (large and positive
+// for a ray along a side), oi = origin * i.
+__device__ __forceinline__ float cube_exit(int x, int y, int z, float k, const RayInv& r)
 {
-    int node = ts.node, leaf = ts.leaf, sp = ts.sp;
-    float bt = ts.bt;
-    uint32_t best = ts.best, best_rec = ts.best_rec;
+    const float tx = fmaf(k, fabsf(r.ix), fmaf((float)x, r.ix, fminf(r.ix, 0.0f) - r.oix));
+    const float ty = fmaf(k, fabsf(r.iy), fmaf((float)y, r.iy, fminf(r.iy, 0.0f) - r.oiy));
+    const float tz = fmaf(k, fabsf(r.iz), fmaf((float)z, r.iz, fminf(r.iz, 0.0f) - r.oiz));
+    return fminf(fminf(tx, ty), tz);
+}
+
+__device__ __forceinline__ uint32_t octant(const RayInv& r)
+{
+    return (__float_as_uint(r.ix) >> 31) | ((__float_as_uint(r.iy) >> 31) << 1) | ((__float_as_uint(r.iz) >> 31) << 2);
+}
+
+// How far a flight of length d from o along dir is clear by the walk grid's
+// empty cubes: true if all of it is; else it is up to t, -1 if it starts
+// outside the grid.  eps: a nudge past a cell's side, in t.
+constexpr uint32_t kNoWalk = 0xFFFFu;   // that -1 where t is kept in 16 bits, in units of walk_unit
+
+__device__ __forceinline__ bool clear_flight(const Scene& sc, float3 o, float3 dir, float d, const RayInv& r, float eps,
+                                             float& t)
+{
+    t = -1.0f;
+    if (!sc.walk_skip) return false;
+    const float gx = fmaf(o.x, sc.grid_inv, sc.grid_off[0]), gy = fmaf(o.y, sc.grid_inv, sc.grid_off[1]),
+                gz = fmaf(o.z, sc.grid_inv, sc.grid_off[2]);
+    const float ux = dir.x * sc.grid_inv, uy = dir.y * sc.grid_inv, uz = dir.z * sc.grid_inv;
+    const uint32_t oct = octant(r);
+    float tc = 0.0f;
+#pragma unroll 1
+    for (int hop = 0; hop < kSafeHops; ++hop) {
+        const int x = (int)fminf(fmaxf(fmaf(tc, ux, gx), 0.5f), sc.walk_max[0]);
+        const int y = (int)fminf(fmaxf(fmaf(tc, uy, gy), 0.5f), sc.walk_max[1]);
+        const int z = (int)fminf(fmaxf(fmaf(tc, uz, gz), 0.5f), sc.walk_max[2]);
+        const uint32_t k = __ldg(&sc.walk_skip[8u * (uint32_t)((z * sc.walk_n[1] + y) * sc.walk_n[0] + x) + oct]);
+        if (k == kCellOut) return hop > 0;   // it has left the grid: nothing is ahead
+        t = tc;
+        if (k == 0u) return false;
+        tc = fmaxf(cube_exit(x, y, z, (float)k, r), tc) + eps;
+        t = tc;
+        if (tc > d) return true;
+    }
+    return false;
+}
+
+// One step of a query's walk through the grid: to the far side of the empty
+// cube ahead, or of an occupied cell, whose sub-tree is descended first.  The
+// triangles' parts reach over their cells by more than the nudge and the
+// rounding here.  The walk is over (the next stack entry follows) once it has
+// left the grid or passed the closest hit.
+__device__ __forceinline__ void walk_step(const Scene& sc, const float4* q, const RayInv& r, float eps, float bt,
+                                          float& t, int& node, int* stack, int& sp)
+{
+    const float4 a = q[0], b = q[1];
+    const int x = (int)fmaf(fmaf(t, b.x, a.x), sc.grid_inv, sc.grid_off[0]);
+    const int y = (int)fmaf(fmaf(t, b.y, a.y), sc.grid_inv, sc.grid_off[1]);
+    const int z = (int)fmaf(fmaf(t, b.z, a.z), sc.grid_inv, sc.grid_off[2]);
+    // (inside the grid by construction; the limit guards the memory)
+    const uint32_t c = min((uint32_t)((z * sc.walk_n[1] + y) * sc.walk_n[0] + x), sc.walk_cells - 1u);
+    const uint32_t k = __ldg(&sc.walk_skip[8u * c + octant(r)]);
+    if (k == 0u) {
+        node = __ldg(&sc.walk_ref[c]);
+        stack[sp++] = kWalk;
+    }
+    t = fmaxf(cube_exit(x, y, z, fmaxf((float)k, 1.0f), r), t) + eps;
+    if (node == kWalk && (k == kCellOut || t > bt)) node = stack[--sp];
+}
+
+// Clusters whose slab the stretch of a ray with t in (0, tmax] may reach (bit
+// c); the slabs are wider than the rounding here.
+__device__ __forceinline__ uint32_t cluster_mask(const Scene& sc, float3 o, float3 d, float tmax)
+{
+    const float t = tmax * kBoxSlack;
+    const float ex = fmaf(t, d.x, o.x), ey = fmaf(t, d.y, o.y), ez = fmaf(t, d.z, o.z);
+    // (fminf and fmaxf skip the NaN of an unlimited ray with d = 0 along the axis)
+    uint32_t m = 0;
+#pragma unroll 1
+    for (int a = 0; a < 3; ++a) {
+        if (!((sc.layer_axes >> a) & 1u)) continue;
+        const float b = pick(a, o.x, o.y, o.z), e = pick(a, ex, ey, ez);
+        const float l = fminf(b, e), h = fmaxf(b, e);
+#pragma unroll
+        for (int c = 0; c < kMaxClusters; ++c)   // unused entries are empty slabs
+            m |= h >= sc.layer_lo[a][c] && l <= sc.layer_hi[a][c] ? 1u << c : 0u;
+    }
+    return m;
+}
+
+
+#ifndef LXO_WALK_MIN
+#define LXO_WALK_MIN 8
+#endif
+#ifndef LXO_NODE_MIN
+#define LXO_NODE_MIN 8
+#endif
+#ifndef LXO_STOP_DIV
+#define LXO_STOP_DIV 2
+#endif
+
+// Lets the queries of a warp run until `need` of its n0 queries in flight have
+// finished (node kDone).  q: the lane's slot.
+template <bool kStats, class Lap>
+__device__ __forceinline__ void run_queries(const Scene& sc, const float4* q, uint32_t skip, const RayInv& r, float eps,
+                                            int n0, int need, Query& cur, int* stack, int* err, Counters& cnt, Lap&& lap)
+{
+    const uint32_t lane = threadIdx.x & 31u;
+    int node = cur.node, sp = cur.sp;
+    float bt = cur.bt, tw = cur.tw;
+    uint32_t rec = cur.rec;
+    int leaf = 0;   // parked leaf (0 = none: reference 0 is an internal node, never a leaf)
+    // Each pass runs the part of the traversal that most lanes wait
+    // for: a leaf's triangles, a step of the walk, a node.  A lane
+    // with a parked leaf walks or descends on until it meets the next.
     while (true) {
-        while (node >= 0) {
-            node_visit(sc, ts.ix, ts.iy, ts.iz, ts.oix, ts.oiy, ts.oiz, bt * kBoxSlack, node, stack, sp, err);
-            if (node < 0 && node != kDone && leaf == 0) {
-                leaf = node;
-                node = stack[--sp];
-            }
-            if (!__any_sync(__activemask(), leaf == 0)) break;
-        }
-        if (node < 0 && node != kDone && leaf == 0) {  // a leaf reference taken from the stack
+        if (leaf == 0 && is_leaf(node)) {
             leaf = node;
             node = stack[--sp];
         }
-        while (leaf != 0) {
-            test_leaf(sc, ts.wr, leaf, ts.skip, bt, best, best_rec, err);
-            leaf = 0;
-            if (node < 0 && node != kDone) {
-                leaf = node;
-                node = stack[--sp];
-            }
+        if (node == kWalk && tw > bt) node = stack[--sp];
+        const int nw = __popc(__ballot_sync(FULL_MASK, node == kWalk));
+        const int nd = __popc(__ballot_sync(FULL_MASK, node >= 0));
+        const int nl = __popc(__ballot_sync(FULL_MASK, leaf != 0));
+        if (nl > 0 && nw < LXO_WALK_MIN && nd < LXO_NODE_MIN) {
+            const int stop = nl / LXO_STOP_DIV;
+            do {
+                if (kStats && lane == 0) cnt.leaf_iters++;
+                if (leaf != 0) {
+                    {
+                    const float4 o = q[0], sh = q[4];   // origin and shear constants wait in the slot
+                    triangle(sc, WRay{o.x, o.y, o.z, sh.x, sh.y, sh.z, cur.kz}, skip, leaf, bt, rec, err);
+                }
+                    if (kStats) {
+                        cnt.q_leaves += leaf == 0;
+                        cnt.tris++;
+                    }
+                }
+            } while (__popc(__ballot_sync(FULL_MASK, leaf != 0)) > stop);
+            lap(cnt.cyc[kCycLeaf], n0);
+        } else if (nw == 0 && nd == 0) {
+            break;
+        } else if (nw >= nd) {
+            const int stop = nw / LXO_STOP_DIV;
+            do {
+                if (kStats && lane == 0) cnt.walk_iters++;
+                if (node == kWalk) {
+                    if (kStats) cnt.walks++;
+                    walk_step(sc, q, r, eps, bt, tw, node, stack, sp);
+                }
+            } while (__popc(__ballot_sync(FULL_MASK, node == kWalk)) > stop);
+            lap(cnt.cyc[kCycNode], n0);
+        } else {
+            const int stop = nd / LXO_STOP_DIV;
+            do {
+                if (kStats && lane == 0) cnt.node_iters++;
+                if (node >= 0) {
+                    if (kStats) cnt.q_nodes++;
+                    node_visit(sc, r, bt * kBoxSlack, node, stack, sp, err);
+                }
+            } while (__popc(__ballot_sync(FULL_MASK, node >= 0)) > stop);
+            lap(cnt.cyc[kCycNode], n0);
         }
-        if (node == kDone) break;
+        if (n0 - __popc(__ballot_sync(FULL_MASK, node != kDone || leaf != 0)) >= need) break;
     }
-    ts.node = node;
-    ts.leaf = leaf;
-    ts.sp = sp;
-    ts.bt = bt;
-    ts.best = best;
-    ts.best_rec = best_rec;
+    // a parked leaf goes back under the part of the query that is left
+    if (leaf != 0) {
+        stack[sp++] = node;
+        node = leaf;
+    }
+    cur.node = node;
+    cur.sp = sp;
+    cur.bt = bt;
+    cur.tw = tw;
+    cur.rec = rec;
 }
 
-__device__ __forceinline__ Hit trav_result(const TravState& ts)
+// ---------------------------------------------------------------------------
+// rays given by the caller
+// ---------------------------------------------------------------------------
+// fewer rays than this: k_trace_few
+constexpr uint32_t kTraceMany = 400000;
+// Few rays: one lane a ray to its end through layers and main tree.  Little
+// code, which is what counts when the kernel lasts as long as a few hundred
+// instruction fetches (1000 rays in the small TPC: 18 us, with the kernel below
+// 41); `width` rays a warp, so that the rays do not wait for one another.
+__global__ void k_trace_few(const __grid_constant__ Scene sc, const float* __restrict__ org,
+                            const float* __restrict__ dir, const uint32_t* __restrict__ skip,
+                            const float* __restrict__ tmax, uint32_t n, int width, uint32_t* __restrict__ hit,
+                            float* __restrict__ t, int* err)
 {
-    return Hit{ts.best, ts.best_rec, ts.best == LXO_NO_HIT ? INFINITY : ts.bt};
-}
-
-__device__ Hit closest_hit(const Scene& sc, float3 o, float3 d, uint32_t skip, float tmax, int* err)
-{
-    TravState ts;
-    int stack[kStackSize];
-    trav_begin(sc, o, d, skip, tmax, ts, stack);
-    trav_run(sc, ts, stack, err);
-    return trav_result(ts);
-}
-
-__global__ void k_trace(const Scene sc, const float* __restrict__ org, const float* __restrict__ dir,
-                        const uint32_t* __restrict__ skip, const float* __restrict__ tmax, uint32_t n,
-                        uint32_t* __restrict__ hit, float* __restrict__ t, int* err)
-{
-    const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
+    const uint64_t i = (uint64_t)(blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * width + (threadIdx.x & 31u);
+    if ((int)(threadIdx.x & 31u) >= width || i >= n) return;
     const float3 o = f3(org[3 * i], org[3 * i + 1], org[3 * i + 2]);
     const float3 d = f3(dir[3 * i], dir[3 * i + 1], dir[3 * i + 2]);
-    const Hit h = closest_hit(sc, o, d, skip ? skip[i] : LXO_NO_HIT, tmax ? tmax[i] : INFINITY, err);
-    hit[i] = h.id;
-    t[i] = h.t;
+    const uint32_t leave_out = skip ? skip[i] : LXO_NO_HIT;
+    const WRay wr = wray_setup(o, d);
+    const RayInv r = ray_inv(sc, o, d);
+    int stack[kStackSize];
+    Query c = begin_query(sc, o, d, wr.kz, tmax ? tmax[i] : INFINITY, (1u << sc.n_clusters) - 1u, -1.0f, stack);
+    int leaf = 0;   // parked leaf
+    // "while-while" with postponed leaves (Aila & Laine, HPG 2009): a lane
+    // that reaches a leaf parks it and descends on until every lane has one
+    while (true) {
+        while (c.node >= 0) {
+            node_visit(sc, r, c.bt * kBoxSlack, c.node, stack, c.sp, err);
+            if (leaf == 0 && is_leaf(c.node)) {
+                leaf = c.node;
+                c.node = stack[--c.sp];
+            }
+            if (!__any_sync(__activemask(), leaf == 0)) break;
+        }
+        if (leaf == 0 && is_leaf(c.node)) {
+            leaf = c.node;
+            c.node = stack[--c.sp];
+        }
+        while (leaf != 0) {
+            do triangle(sc, wr, leave_out, leaf, c.bt, c.rec, err); while (leaf != 0);
+            if (is_leaf(c.node)) {
+                leaf = c.node;
+                c.node = stack[--c.sp];
+            }
+        }
+        if (c.node == kDone) break;
+    }
+    hit[i] = c.rec == LXO_NO_HIT ? LXO_NO_HIT : __float_as_uint(__ldg(sc.tris + 3 * (size_t)c.rec + 2).y);
+    t[i] = c.rec == LXO_NO_HIT ? INFINITY : c.bt;
+}
+
+// Many rays.  A warp looks at 32 rays at a time: those whose whole flight the empty cubes
+// clear are answered at once, the others wait in a ring of the warp's own,
+// from which its lanes take their next ray when half of those in flight have
+// finished.  What bounds it is the divergence of the queries (a lane a ray to
+// the end of the warp's slowest, whole trees searched: 397 us for 2e6 rays
+// with free-flight limits in the DARWIN-scale mesh; now 251 us).
+constexpr int kTraceThreads = 128, kTraceCtas = 9, kTraceWarps = kTraceThreads / 32, kTraceRing = 64;
+
+__global__ void __launch_bounds__(kTraceThreads, kTraceCtas)
+    k_trace(const __grid_constant__ Scene sc, const float* __restrict__ org, const float* __restrict__ dir,
+            const uint32_t* __restrict__ skip, const float* __restrict__ tmax, uint32_t n,
+            uint32_t* __restrict__ hit, float* __restrict__ t, int* err)
+{
+    __shared__ float4 s_slot[kTraceThreads * kSlotF4];
+    __shared__ uint2 s_ring[kTraceWarps][kTraceRing];   // ray, layers | clear part of its flight << 16 (1 / 64 cells)
+    float4* q = s_slot + kSlotF4 * threadIdx.x;
+    uint2* ring = s_ring[threadIdx.x >> 5];
+    const uint32_t lane = threadIdx.x & 31u;
+    const uint64_t stride = (uint64_t)gridDim.x * kTraceWarps * 32u;
+    uint64_t next = ((uint64_t)blockIdx.x * kTraceWarps + (threadIdx.x >> 5)) * 32u;
+    uint32_t head = 0, tail = 0;   // ring entries taken and put, warp-uniform
+    uint32_t ray = 0;
+    bool have = false;
+    uint32_t leave_out = 0;        // triangle id not to be hit
+    float eps = 0.0f;
+    RayInv r{};
+    Query cur{kDone, 1, 0, 0.0f, 0.0f, LXO_NO_HIT};
+    int stack[kStackSize];
+    Counters cnt{};
+    auto lap = [](unsigned long long&, int) {};
+    while (true) {
+        const uint32_t idle = __ballot_sync(FULL_MASK, !have);
+        while (next < n && tail - head < (uint32_t)__popc(idle)) {   // at most 31 + 32 entries
+            const uint64_t i = next + lane;
+            bool wait = false;
+            uint32_t word = 0;
+            if (i < n) {
+                const float3 o = f3(org[3 * i], org[3 * i + 1], org[3 * i + 2]);
+                const float3 d = f3(dir[3 * i], dir[3 * i + 1], dir[3 * i + 2]);
+                const float tm = tmax ? tmax[i] : INFINITY;
+                const RayInv ri = ray_inv(sc, o, d);
+                // directions of any length: t of one cell along the main
+                // axis; the main tree is searched where the numbers might not
+                // carry the walk (0, infinite, NaN)
+                const float cell = fminf(fminf(fabsf(ri.ix), fabsf(ri.iy)), fabsf(ri.iz));
+                float clear_to = -1.0f;
+                bool clear = false;
+                if (cell > 1e-18f * sc.grid_h && cell < 1e18f * sc.grid_h)
+                    clear = clear_flight(sc, o, d, tm, ri, 0.002f * cell, clear_to);
+                const uint32_t layers = cluster_mask(sc, o, d, tm);
+                wait = tm > 0.0f && !(clear && layers == 0u);
+                if (!wait) {
+                    hit[i] = LXO_NO_HIT;
+                    t[i] = INFINITY;
+                }
+                word = layers | ((clear_to >= 0.0f ? min((uint32_t)__fdividef(64.0f * clear_to, cell), kNoWalk - 1u)
+                                                   : kNoWalk) << 16);
+            }
+            const uint32_t m = __ballot_sync(FULL_MASK, wait);
+            if (wait) ring[(tail + __popc(m & ((1u << lane) - 1u))) % kTraceRing] = make_uint2((uint32_t)i, word);
+            tail += __popc(m);
+            next += stride;
+        }
+        __syncwarp();
+        const uint32_t take = min(tail - head, (uint32_t)__popc(idle));
+        const uint32_t rank = __popc(idle & ((1u << lane) - 1u));
+        if (((idle >> lane) & 1u) && rank < take) {
+            const uint2 e = ring[(head + rank) % kTraceRing];
+            ray = e.x;
+            const float3 o = f3(org[3ull * ray], org[3ull * ray + 1], org[3ull * ray + 2]);
+            const float3 d = f3(dir[3ull * ray], dir[3ull * ray + 1], dir[3ull * ray + 2]);
+            leave_out = skip ? skip[ray] : LXO_NO_HIT;
+            r = ray_inv(sc, o, d);
+            const float cell = fminf(fminf(fabsf(r.ix), fabsf(r.iy)), fabsf(r.iz));
+            eps = 0.002f * cell;
+            float3 sh;
+            const int kz = shear(d, sh);
+            q[0] = make_float4(o.x, o.y, o.z, 0.0f);
+            q[1] = make_float4(d.x, d.y, d.z, 0.0f);
+            q[4] = make_float4(sh.x, sh.y, sh.z, 0.0f);
+            const uint32_t units = e.y >> 16;
+            cur = begin_query(sc, o, d, kz, tmax ? tmax[ray] : INFINITY, e.y & 0xFFu,
+                              units != kNoWalk ? (float)units * (cell * (1.0f / 64.0f)) : -1.0f, stack);
+            have = true;
+        }
+        head += take;
+        const int n0 = __popc(__ballot_sync(FULL_MASK, have));
+        if (n0 == 0) break;   // then the ring is empty and no ray is left
+        run_queries<false>(sc, q, leave_out, r, eps, n0, max(1, n0 / 2), cur, stack, err, cnt, lap);
+        if (have && cur.node == kDone) {
+            hit[ray] = cur.rec == LXO_NO_HIT ? LXO_NO_HIT : __float_as_uint(__ldg(sc.tris + 3 * (size_t)cur.rec + 2).y);
+            t[ray] = cur.rec == LXO_NO_HIT ? INFINITY : cur.bt;
+            have = false;
+        }
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -967,23 +1188,12 @@ __device__ __forceinline__ int surface_event(const PropParams& p, Photon& ph, fl
 #ifndef LXO_LEAVE_DIV
 #define LXO_LEAVE_DIV 2
 #endif
-#ifndef LXO_WALK_MIN
-#define LXO_WALK_MIN 8
-#endif
-#ifndef LXO_NODE_MIN
-#define LXO_NODE_MIN 8
-#endif
-#ifndef LXO_STOP_DIV
-#define LXO_STOP_DIV 2
-#endif
 #ifndef LXO_BATCH_MIN
 #define LXO_BATCH_MIN 28
 #endif
 constexpr int kPoolThreads = LXO_POOL_THREADS, kPoolCtas = LXO_POOL_CTAS;
 constexpr int kPoolWarps = kPoolThreads / 32;
 constexpr int kMaxSlots = 1024;       // 32 columns of 32
-constexpr int kSlotF4 = 5;            // float4 per slot
-constexpr uint32_t kNoTri = 0x0FFFFFFFu;  // "no triangle" in 28 bits (ids stay below 2^28 - 1)
 constexpr uint32_t kPollLimit = 1u << 20;   // a warp that has found nothing so often leaves (never a lost photon: it holds none)
 
 // Where a slot's photon waits.
@@ -1076,104 +1286,6 @@ __device__ __forceinline__ void step_histogram(const PropParams& p, int medium, 
     atomicAdd(&p.out.stats[9 + 10 * m + 9], (unsigned long long)dl);
 }
 
-// Distance at which a ray leaves the cube of k cells (an octant's) that starts
-// with its cell (x, y, z): in grid space, i = 1 / direction (large and positive
-// for a ray along a side), oi = origin * i.
-__device__ __forceinline__ float cube_exit(int x, int y, int z, float k, float ix, float iy, float iz, float oix,
-                                           float oiy, float oiz)
-{
-    const float tx = fmaf(k, fabsf(ix), fmaf((float)x, ix, fminf(ix, 0.0f) - oix));
-    const float ty = fmaf(k, fabsf(iy), fmaf((float)y, iy, fminf(iy, 0.0f) - oiy));
-    const float tz = fmaf(k, fabsf(iz), fmaf((float)z, iz, fminf(iz, 0.0f) - oiz));
-    return fminf(fminf(tx, ty), tz);
-}
-
-__device__ __forceinline__ uint32_t octant(float ix, float iy, float iz)
-{
-    return (__float_as_uint(ix) >> 31) | ((__float_as_uint(iy) >> 31) << 1) | ((__float_as_uint(iz) >> 31) << 2);
-}
-
-// How far a flight of length d from o along dir is clear by the walk grid's
-// empty cubes: true if all of it is; else `units` of walk_unit are clear,
-// kNoWalk if it starts outside the grid.
-constexpr uint32_t kNoWalk = 0xFFFFu;
-
-__device__ __forceinline__ bool clear_flight(const Scene& sc, float3 o, float3 dir, float d, uint32_t& units)
-{
-    units = kNoWalk;
-    if (!sc.walk_skip) return false;
-    const float gx = fmaf(o.x, sc.grid_inv, sc.grid_off[0]), gy = fmaf(o.y, sc.grid_inv, sc.grid_off[1]),
-                gz = fmaf(o.z, sc.grid_inv, sc.grid_off[2]);
-    const float ix = fast_inv(dir.x) * sc.grid_h, iy = fast_inv(dir.y) * sc.grid_h, iz = fast_inv(dir.z) * sc.grid_h;
-    const float ux = dir.x * sc.grid_inv, uy = dir.y * sc.grid_inv, uz = dir.z * sc.grid_inv;
-    const uint32_t oct = octant(ix, iy, iz);
-    float t = 0.0f;
-    bool clear = false;
-#pragma unroll 1
-    for (int hop = 0; hop < kSafeHops; ++hop) {
-        const int x = (int)fminf(fmaxf(fmaf(t, ux, gx), 0.5f), sc.walk_max[0]);
-        const int y = (int)fminf(fmaxf(fmaf(t, uy, gy), 0.5f), sc.walk_max[1]);
-        const int z = (int)fminf(fmaxf(fmaf(t, uz, gz), 0.5f), sc.walk_max[2]);
-        const uint32_t k = __ldg(&sc.walk_skip[8u * (uint32_t)((z * sc.walk_n[1] + y) * sc.walk_n[0] + x) + oct]);
-        if (k == kCellOut) {
-            if (hop == 0) return false;
-            clear = true;   // it has left the grid: nothing is ahead
-            break;
-        }
-        if (k == 0u) break;
-        t = fmaxf(cube_exit(x, y, z, (float)k, ix, iy, iz, gx * ix, gy * iy, gz * iz), t) + sc.walk_eps;
-        if (t > d) {
-            clear = true;
-            break;
-        }
-    }
-    units = min((uint32_t)(t * sc.walk_per_mm), kNoWalk - 1u);
-    return clear;
-}
-
-// One step of a query's walk through the grid: to the far side of the empty
-// cube ahead, or of an occupied cell, whose sub-tree is descended first.  The
-// triangles' parts reach over their cells by more than the nudge and the
-// rounding here.  The walk is over (the next stack entry follows) once it has
-// left the grid or passed the closest hit.
-__device__ __forceinline__ void walk_step(const Scene& sc, const float4* q, float ix, float iy, float iz, float oix,
-                                          float oiy, float oiz, float bt, float& t, int& node, int* stack, int& sp)
-{
-    const float4 a = q[0], b = q[1];
-    const int x = (int)fmaf(fmaf(t, b.x, a.x), sc.grid_inv, sc.grid_off[0]);
-    const int y = (int)fmaf(fmaf(t, b.y, a.y), sc.grid_inv, sc.grid_off[1]);
-    const int z = (int)fmaf(fmaf(t, b.z, a.z), sc.grid_inv, sc.grid_off[2]);
-    // (inside the grid by construction; the limit guards the memory)
-    const uint32_t c = min((uint32_t)((z * sc.walk_n[1] + y) * sc.walk_n[0] + x), sc.walk_cells - 1u);
-    const uint32_t k = __ldg(&sc.walk_skip[8u * c + octant(ix, iy, iz)]);
-    if (k == 0u) {
-        node = __ldg(&sc.walk_ref[c]);
-        stack[sp++] = kWalk;
-    }
-    t = fmaxf(cube_exit(x, y, z, fmaxf((float)k, 1.0f), ix, iy, iz, oix, oiy, oiz), t) + sc.walk_eps;
-    if (node == kWalk && (k == kCellOut || t > bt)) node = stack[--sp];
-}
-
-// Clusters whose slab the stretch of a ray with t in (0, tmax] may reach (bit
-// c); the slabs are wider than the rounding here.
-__device__ __forceinline__ uint32_t cluster_mask(const Scene& sc, float3 o, float3 d, float tmax)
-{
-    const float t = tmax * kBoxSlack;
-    const float ex = fmaf(t, d.x, o.x), ey = fmaf(t, d.y, o.y), ez = fmaf(t, d.z, o.z);
-    // (fminf and fmaxf skip the NaN of an unlimited ray with d = 0 along the axis)
-    uint32_t m = 0;
-#pragma unroll 1
-    for (int a = 0; a < 3; ++a) {
-        if (!((sc.layer_axes >> a) & 1u)) continue;
-        const float b = pick(a, o.x, o.y, o.z), e = pick(a, ex, ey, ez);
-        const float l = fminf(b, e), h = fmaxf(b, e);
-#pragma unroll
-        for (int c = 0; c < kMaxClusters; ++c)   // unused entries are empty slabs
-            m |= h >= sc.layer_lo[a][c] && l <= sc.layer_hi[a][c] ? 1u << c : 0u;
-    }
-    return m;
-}
-
 // A slot: five float4.
 //   [0] position, flight length (sign bit: absorption at its end) or hit distance
 //   [1] direction, a word: ready: axis kz | cluster mask << 2 | clear units << 16;  after the
@@ -1222,11 +1334,9 @@ __global__ void __launch_bounds__(kPoolThreads, kPoolCtas) k_propagate(const __g
     const uint32_t lt_mask = (1u << lane) - 1u;
     const int warp = threadIdx.x >> 5;
     const int turn = warp & 31;
-    // the lane's query in flight: its slot (-1 none), closest hit so far and
-    // traversal state (kDone: not started); its stack in local memory
-    int slot = -1, node = kDone, sp = 1, kz = 0;
-    float bt = 0.0f, tw = 0.0f;
-    uint32_t rec = LXO_NO_HIT;
+    // the lane's query in flight: its slot (-1 none) and state; its stack in local memory
+    int slot = -1;
+    Query cur{kDone, 1, 0, 0.0f, 0.0f, LXO_NO_HIT};
     int stack[kStackSize];
     uint32_t polls = 0;
     Counters cnt{};
@@ -1289,100 +1399,28 @@ __global__ void __launch_bounds__(kPoolThreads, kPoolCtas) k_propagate(const __g
             const int n0 = __popc(__ballot_sync(FULL_MASK, slot >= 0));
             if (n0 == 0) continue;
             const float4* q = s_pool + kSlotF4 * max(slot, 0);
-            float ix = 0.0f, iy = 0.0f, iz = 0.0f, oix = 0.0f, oiy = 0.0f, oiz = 0.0f;
-            uint32_t clusters = 0;
+            RayInv ray{};
             if (slot >= 0) {
                 const float4 a = q[0], b = q[1];
-                ix = fast_inv(b.x) * p.sc.grid_h;
-                iy = fast_inv(b.y) * p.sc.grid_h;
-                iz = fast_inv(b.z) * p.sc.grid_h;
-                oix = fmaf(a.x, p.sc.grid_inv, p.sc.grid_off[0]) * ix;
-                oiy = fmaf(a.y, p.sc.grid_inv, p.sc.grid_off[1]) * iy;
-                oiz = fmaf(a.z, p.sc.grid_inv, p.sc.grid_off[2]) * iz;
+                const float3 o = f3(a.x, a.y, a.z), d = f3(b.x, b.y, b.z);
+                ray = ray_inv(p.sc, o, d);
                 if (fresh) {
-                    const uint32_t kw = __float_as_uint(b.w);
-                    kz = (int)(kw & 3u);
-                    clusters = (kw >> 2) & 0xFFu;
-                    bt = fabsf(a.w);
-                    rec = LXO_NO_HIT;
-                    stack[0] = kDone;
-                    sp = 1;
-                    if (clusters)
-                        enter_clusters(p.sc, clusters, f3(a.x, a.y, a.z), f3(b.x, b.y, b.z), bt, stack, sp);
-                    // in the grid: the walk from where the flight is clear to;
-                    // else the main tree
-                    const uint32_t units = kw >> 16;
-                    tw = (float)units * p.sc.walk_unit;
-                    node = units != kNoWalk ? kWalk : p.sc.main_root;
-                    if (node == kEmptyChild) node = stack[--sp];
+                    const uint32_t kw = __float_as_uint(b.w), units = kw >> 16;
+                    cur = begin_query(p.sc, o, d, (int)(kw & 3u), fabsf(a.w), (kw >> 2) & 0xFFu,
+                                      units != kNoWalk ? (float)units * p.sc.walk_unit : -1.0f, stack);
                 }
             }
             __syncwarp();
             lap(cnt.cyc[kCycBegin], n0);
             if (kStats && lane == 0) cnt.entries++;
-            int leaf = 0;   // parked leaf (0 = none: reference 0 is an internal node, never a leaf)
             const int need = max(1, n0 / LXO_LEAVE_DIV);
             const uint32_t skip = __float_as_uint(q[3].w) & kNoTri;
-            // Each pass runs the part of the traversal that most lanes wait
-            // for: a leaf's triangles, a step of the walk, a node.  A lane
-            // with a parked leaf walks or descends on until it meets the next.
-            while (true) {
-                if (leaf == 0 && is_leaf(node)) {
-                    leaf = node;
-                    node = stack[--sp];
-                }
-                if (node == kWalk && tw > bt) node = stack[--sp];
-                const int nw = __popc(__ballot_sync(FULL_MASK, node == kWalk));
-                const int nd = __popc(__ballot_sync(FULL_MASK, node >= 0));
-                const int nl = __popc(__ballot_sync(FULL_MASK, leaf != 0));
-                if (nl > 0 && nw < LXO_WALK_MIN && nd < LXO_NODE_MIN) {
-                    const int stop = nl / LXO_STOP_DIV;
-                    do {
-                        if (kStats && lane == 0) cnt.leaf_iters++;
-                        if (leaf != 0) {
-                            slot_triangle(p.sc, q, kz, skip, leaf, bt, rec, p.err);
-                            if (kStats) {
-                                cnt.q_leaves += leaf == 0;
-                                cnt.tris++;
-                            }
-                        }
-                    } while (__popc(__ballot_sync(FULL_MASK, leaf != 0)) > stop);
-                    lap(cnt.cyc[kCycLeaf], n0);
-                } else if (nw == 0 && nd == 0) {
-                    break;
-                } else if (nw >= nd) {
-                    const int stop = nw / LXO_STOP_DIV;
-                    do {
-                        if (kStats && lane == 0) cnt.walk_iters++;
-                        if (node == kWalk) {
-                            if (kStats) cnt.walks++;
-                            walk_step(p.sc, q, ix, iy, iz, oix, oiy, oiz, bt, tw, node, stack, sp);
-                        }
-                    } while (__popc(__ballot_sync(FULL_MASK, node == kWalk)) > stop);
-                    lap(cnt.cyc[kCycNode], n0);
-                } else {
-                    const int stop = nd / LXO_STOP_DIV;
-                    do {
-                        if (kStats && lane == 0) cnt.node_iters++;
-                        if (node >= 0) {
-                            if (kStats) cnt.q_nodes++;
-                            node_visit(p.sc, ix, iy, iz, oix, oiy, oiz, bt * kBoxSlack, node, stack, sp, p.err);
-                        }
-                    } while (__popc(__ballot_sync(FULL_MASK, node >= 0)) > stop);
-                    lap(cnt.cyc[kCycNode], n0);
-                }
-                if (n0 - __popc(__ballot_sync(FULL_MASK, node != kDone || leaf != 0)) >= need) break;
-            }
-            // a parked leaf goes back under the part of the query that is left
-            if (leaf != 0) {
-                stack[sp++] = node;
-                node = leaf;
-            }
-            const bool done = slot >= 0 && node == kDone;
+            run_queries<kStats>(p.sc, q, skip, ray, p.sc.walk_eps, n0, need, cur, stack, p.err, cnt, lap);
+            const bool done = slot >= 0 && cur.node == kDone;
             if (done) {
                 float4* w = s_pool + kSlotF4 * slot;
-                if (rec != LXO_NO_HIT) w[0].w = bt;
-                w[1].w = __uint_as_float(rec);
+                if (cur.rec != LXO_NO_HIT) w[0].w = cur.bt;
+                w[1].w = __uint_as_float(cur.rec);
             }
             if (kStats && done) {
                 step_histogram(p, (int)(__float_as_uint(q[3].w) >> 28), cnt.q_nodes, cnt.q_leaves);
@@ -1392,7 +1430,7 @@ __global__ void __launch_bounds__(kPoolThreads, kPoolCtas) k_propagate(const __g
             }
             __threadfence_block();
             if (done) {
-                put(s_set[rec != LXO_NO_HIT ? kSurf : kBulk], slot);
+                put(s_set[cur.rec != LXO_NO_HIT ? kSurf : kBulk], slot);
                 slot = -1;
             }
             __syncwarp();
@@ -1462,15 +1500,16 @@ __global__ void __launch_bounds__(kPoolThreads, kPoolCtas) k_propagate(const __g
             const float d = fminf(sd.d_abs, sd.d_ray);
             uint32_t word = LXO_NO_HIT;
             float3 sh = f3(0.0f, 0.0f, 0.0f);
-            uint32_t units;
+            float clear_to;
             const uint32_t clusters = cluster_mask(p.sc, ph.pos, ph.dir, d);
-            const bool clear = clear_flight(p.sc, ph.pos, ph.dir, d, units);
+            const bool clear = clear_flight(p.sc, ph.pos, ph.dir, d, ray_inv(p.sc, ph.pos, ph.dir), p.sc.walk_eps, clear_to);
             if (clear && clusters == 0u) {
                 to = kBulk;
                 if (kStats) step_histogram(p, ph.medium, 0, 0);
             } else {
                 to = clusters ? kReadyLayer : kReady;
                 const int k = shear(ph.dir, sh);
+                const uint32_t units = clear_to >= 0.0f ? min((uint32_t)(clear_to * p.sc.walk_per_mm), kNoWalk - 1u) : kNoWalk;
                 word = (uint32_t)k | (clusters << 2) | (units << 16);
             }
             const uint32_t ab = sd.d_abs <= sd.d_ray ? 0x80000000u : 0u;
@@ -1522,8 +1561,18 @@ cudaError_t launch_trace(const Scene& sc, const float* org, const float* dir, co
                          const float* tmax, uint32_t n, uint32_t* hit, float* t, int* err, cudaStream_t st)
 {
     if (n == 0) return cudaSuccess;
-    const int threads = 128;
-    k_trace<<<(n + threads - 1) / threads, threads, 0, st>>>(sc, org, dir, skip, tmax, n, hit, t, err);
+    int dev = 0, sms = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    if (n < kTraceMany) {
+        const uint64_t warps = (uint64_t)sms * 16u;
+        const int width = (int)std::min<uint64_t>(32u, (n + warps - 1) / warps);
+        const unsigned blocks = (unsigned)(((n + width - 1u) / width + kTraceWarps - 1) / kTraceWarps);
+        k_trace_few<<<blocks, kTraceThreads, 0, st>>>(sc, org, dir, skip, tmax, n, width, hit, t, err);
+        return cudaGetLastError();
+    }
+    k_trace<<<(unsigned)(sms * kTraceCtas), kTraceThreads, 0, st>>>(sc, org, dir, skip, tmax, n, hit, t, err);
     return cudaGetLastError();
 }
 

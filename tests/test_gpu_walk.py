@@ -1,7 +1,11 @@
-"""The photon kernel's own route to the closest hit (flights cleared by empty
-cubes, the walk through the grid, planar layers entered by their cells) against
-the plain tree search of lxo_trace_rays, ray by ray, and its pool of photon
-slots at sizes around a lane, a warp, a CTA and the whole GPU.
+"""The route to the closest hit (flights cleared by empty cubes, the walk
+through the grid, planar layers entered by their cells) against the search of
+the main tree, ray by ray, in lxo_trace_rays and in the photon kernel, and the
+kernel's pool of photon slots at sizes around a lane, a warp, a CTA and the
+whole GPU.
+
+Directions 2^64 long are left to the main tree: every number of the exact
+triangle test then scales by a power of two, so hits and t stay the same.
 
 Every triangle absorbs and no medium scatters, so a photon ends at its first
 hit with its direction unchanged: its time is t n / c for the t of the same
@@ -70,6 +74,29 @@ def test_first_hits_match_the_tree_search(name):
     assert np.array_equal(fate, np.where(hit >= 0, 3, 4))   # absorbed by the surface, or escaped
     assert np.array_equal(time[hit >= 0], (t * N_OVER_C)[hit >= 0])
     assert int(out["fates"][:7].sum()) == n
+
+
+@pytest.mark.parametrize("name", DETECTORS)
+@pytest.mark.parametrize("n", [1, 33, 40_000])
+def test_walk_matches_the_main_tree(name, n):
+    import torch
+    from paper_2203_14354_gb300 import Tracker
+    det = DETECTORS[name]()
+    trk = Tracker(det)
+    org, d, _ = [torch.from_numpy(x).cuda() for x in rays(det, n, seed=5 + n)]
+    far = 2.0 ** 64
+    rng = np.random.default_rng(n)
+    size = float(np.ptp(det.verts, axis=0).max())
+    tmax = torch.from_numpy(rng.exponential(0.3 * size, n).astype(np.float32)).cuda()
+    tmax[::7] = float("inf")
+    tmax[::11] = 0.0
+    hit, _ = trk.trace_rays(org, d)
+    for scale in (1.0, 0.125, 1024.0):   # directions of any length
+        for skip, tm in ((None, None), (None, tmax), (hit, None), (hit, tmax)):
+            a = trk.trace_rays(org, d * scale, skip, None if tm is None else tm / scale)
+            b = trk.trace_rays(org, d * far, skip, None if tm is None else tm / far)
+            assert torch.equal(a[0], b[0])
+            assert torch.equal(a[1] * scale, b[1] * far)
 
 
 def test_pool_sizes():
