@@ -730,20 +730,18 @@ __device__ __forceinline__ bool inside_poly(const SourceDev& s, float x, float y
 // position from the event's point / segment / ball.
 // Emission delay of the scintillation time profile (Sec. 2.2, Table 2): a
 // mixture of two exponentials, from its own draw of the source step.
-__device__ __forceinline__ float emission_delay(const PropParams& p, uint64_t pid, const TimeProfile& tp)
+__device__ __forceinline__ float emission_delay(const U4& u, const TimeProfile& tp)
 {
     if (tp.tau_s == 0.0f && tp.tau_t == 0.0f) return 0.0f;
-    const U4 u = draw4<1>(p.seed, pid, kSourceStep, 0xFFFFFFFFu);
     const float tau = u.u0 < tp.f_s ? tp.tau_s : tp.tau_t;
     return -tau * logf(u.u1);
 }
 
 // Wavelength from the Gaussian emission spectrum (Sec. 2.2, Table 2): the
 // Box-Muller transform of the last two uniforms of the emission draw.
-__device__ __forceinline__ float emission_wavelength(const PropParams& p, uint64_t pid, const Spectrum& sp)
+__device__ __forceinline__ float emission_wavelength(const U4& u, const Spectrum& sp)
 {
     if (sp.sigma == 0.0f) return sp.mean;
-    const U4 u = draw4<1>(p.seed, pid, kSourceStep, 0xFFFFFFFFu);
     float s, c;
     sincospif(2.0f * u.u3, &s, &c);
     return fmaf(sp.sigma, sqrtf(-2.0f * logf(u.u2)) * c, sp.mean);
@@ -764,7 +762,18 @@ __device__ __forceinline__ float n_over_c_at(const DevMaterial& m, float wl)
     return kSpectral ? fmaf(m.dn_over_c, wl - LXO_REF_WAVELENGTH_NM, m.n_over_c) : m.n_over_c;
 }
 
-__device__ Photon make_event_photon(const PropParams& p, uint64_t idx)
+// The emission draw, if the time profile or the spectrum needs it.
+template <int kRounds>
+__device__ __forceinline__ U4 emission_draw(const PropParams& p, uint64_t pid, const TimeProfile& tp, const Spectrum& sp,
+                                            bool want_wl)
+{
+    if (tp.tau_s == 0.0f && tp.tau_t == 0.0f && (!want_wl || sp.sigma == 0.0f)) return U4{0.5f, 0.5f, 0.5f, 0.5f};
+    return draw4<kRounds>(p.seed, pid, kSourceStep, 0xFFFFFFFFu);
+}
+
+// kRounds: see philox4x32_10; want_wl: the wavelength is wanted.
+template <int kRounds>
+__device__ Photon make_event_photon(const PropParams& p, uint64_t idx, bool want_wl)
 {
     uint32_t lo = 0, hi = p.n_events;  // find e with prefix[e] <= idx < prefix[e+1]
     while (hi - lo > 1) {
@@ -775,11 +784,12 @@ __device__ Photon make_event_photon(const PropParams& p, uint64_t idx)
     Photon ph;
     ph.pid = ((uint64_t)(p.first_event + lo) << 32) | (uint64_t)(idx - __ldg(&p.ev_prefix[lo]));
     ph.medium = ev.medium;
-    ph.time = ev.t0 + emission_delay(p, ph.pid, ev.prof);
-    ph.wl = p.spectral ? emission_wavelength(p, ph.pid, ev.spec) : 0.0f;
+    const U4 em = emission_draw<kRounds>(p, ph.pid, ev.prof, ev.spec, want_wl);
+    ph.time = ev.t0 + emission_delay(em, ev.prof);
+    ph.wl = want_wl ? emission_wavelength(em, ev.spec) : 0.0f;
     ph.last = LXO_NO_HIT;
     ph.step = 0;
-    const U4 u = draw4<1>(p.seed, ph.pid, kSourceStep, 0);
+    const U4 u = draw4<kRounds>(p.seed, ph.pid, kSourceStep, 0);
     const float c = 2.0f * u.u0 - 1.0f, sn = sqrtf(fmaxf(0.0f, 1.0f - c * c));
     float sp, cp;
     sincospif(2.0f * u.u1, &sp, &cp);
@@ -793,7 +803,7 @@ __device__ Photon make_event_photon(const PropParams& p, uint64_t idx)
         if (ev.kind == LXO_SRC_BALL) {
 #pragma unroll 1
             for (int tr = 0; tr < kMaxTries; ++tr) {
-                const U4 w = draw4<1>(p.seed, ph.pid, kSourceStep, 1 + tr);
+                const U4 w = draw4<kRounds>(p.seed, ph.pid, kSourceStep, 1 + tr);
                 const float x = ev.radius * (2.0f * w.u0 - 1.0f), y = ev.radius * (2.0f * w.u1 - 1.0f),
                             z = ev.radius * (2.0f * w.u2 - 1.0f);
                 if (x * x + y * y + z * z <= ev.radius * ev.radius) {
@@ -806,15 +816,17 @@ __device__ Photon make_event_photon(const PropParams& p, uint64_t idx)
     return ph;
 }
 
-__device__ Photon make_photon(const PropParams& p, uint64_t idx)
+template <int kRounds>
+__device__ Photon make_photon(const PropParams& p, uint64_t idx, bool want_wl)
 {
-    if (p.n_events) return make_event_photon(p, idx);
+    if (p.n_events) return make_event_photon<kRounds>(p, idx, want_wl);
     const SourceDev& s = p.src;
     Photon ph;
     ph.pid = p.base + idx;
     ph.medium = s.medium;
-    ph.time = s.t0 + emission_delay(p, ph.pid, s.prof);
-    ph.wl = p.spectral ? emission_wavelength(p, ph.pid, s.spec) : 0.0f;
+    const U4 em = emission_draw<kRounds>(p, ph.pid, s.prof, s.spec, want_wl);
+    ph.time = s.t0 + emission_delay(em, s.prof);
+    ph.wl = want_wl ? emission_wavelength(em, s.spec) : 0.0f;
     ph.last = LXO_NO_HIT;
     ph.step = 0;
     if (s.kind == LXO_SRC_EXPLICIT) {
@@ -824,7 +836,7 @@ __device__ Photon make_photon(const PropParams& p, uint64_t idx)
         ph.pol = normalize(e - dot(e, ph.dir) * ph.dir);
         return ph;
     }
-    const U4 u = draw4<1>(p.seed, ph.pid, kSourceStep, 0);
+    const U4 u = draw4<kRounds>(p.seed, ph.pid, kSourceStep, 0);
     const float c = 2.0f * u.u0 - 1.0f, sn = sqrtf(fmaxf(0.0f, 1.0f - c * c));
     float sp, cp;
     sincospif(2.0f * u.u1, &sp, &cp);
@@ -839,7 +851,7 @@ __device__ Photon make_photon(const PropParams& p, uint64_t idx)
         ph.pos = f3(s.center[0], s.center[1], s.center[2]);
 #pragma unroll 1
         for (int tr = 0; tr < kMaxTries; ++tr) {
-            const U4 w = draw4<1>(p.seed, ph.pid, kSourceStep, 1 + tr);
+            const U4 w = draw4<kRounds>(p.seed, ph.pid, kSourceStep, 1 + tr);
             const float x = s.radius * (2.0f * w.u0 - 1.0f), y = s.radius * (2.0f * w.u1 - 1.0f),
                         z = s.radius * (2.0f * w.u2 - 1.0f);
             if (x * x + y * y + z * z <= s.radius * s.radius) {
@@ -851,7 +863,7 @@ __device__ Photon make_photon(const PropParams& p, uint64_t idx)
         ph.pos = f3(0.0f, 0.0f, s.z_min + u.u3 * (s.z_max - s.z_min));
 #pragma unroll 1
         for (int tr = 0; tr < kMaxTries; ++tr) {
-            const U4 w = draw4<1>(p.seed, ph.pid, kSourceStep, 1 + tr);
+            const U4 w = draw4<kRounds>(p.seed, ph.pid, kSourceStep, 1 + tr);
             float r = s.radius * sqrtf(w.u0), sa, ca;
             sincospif(2.0f * w.u1, &sa, &ca);
             if (inside_poly(s, r * ca, r * sa, w.u1)) {
@@ -871,17 +883,23 @@ __device__ Photon make_photon(const PropParams& p, uint64_t idx)
     return ph;
 }
 
+// Bound by issue slots (three generator calls, six sines and cosines, two
+// logarithms a photon), so the stores are plain: through shared memory, in full
+// lines, 4e6 photons with time profile and spectrum took 98 us, so 90 before
+// the two emission draws became one and 84 now.
+constexpr int kSampleThreads = 128;
+
 __global__ void k_sample_source(const __grid_constant__ PropParams p, float* pos, float* dir, float* pol,
                                 float* time, float* wavelength)
 {
     const uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= p.n) return;
-    const Photon ph = make_photon(p, i);
+    const Photon ph = make_photon<10>(p, i, wavelength != nullptr);
     pos[3 * i] = ph.pos.x; pos[3 * i + 1] = ph.pos.y; pos[3 * i + 2] = ph.pos.z;
     dir[3 * i] = ph.dir.x; dir[3 * i + 1] = ph.dir.y; dir[3 * i + 2] = ph.dir.z;
     pol[3 * i] = ph.pol.x; pol[3 * i + 1] = ph.pol.y; pol[3 * i + 2] = ph.pol.z;
     if (time) time[i] = ph.time;
-    if (wavelength) wavelength[i] = emission_wavelength(p, ph.pid, p.src.spec);
+    if (wavelength) wavelength[i] = ph.wl;
 }
 
 // ---------------------------------------------------------------------------
@@ -1466,7 +1484,7 @@ __global__ void __launch_bounds__(kPoolThreads, kPoolCtas) k_propagate(const __g
             }
             const int rank = __popc(members & lt_mask);
             if (s >= 0 && rank < avail) {
-                ph = make_photon(p, base + rank);
+                ph = make_photon<1>(p, base + rank, p.spectral != 0);
                 if (kAdjoint)
                     for (int k = 0; k < p.adj_k; ++k) tl[k] = 0.0f;
                 alive = true;
@@ -1580,9 +1598,8 @@ cudaError_t launch_sample_source(const PropParams& p, float* pos, float* dir, fl
                                  float* wavelength, cudaStream_t st)
 {
     if (p.n == 0) return cudaSuccess;
-    const int threads = 128;
-    const uint64_t blocks = (p.n + threads - 1) / threads;
-    k_sample_source<<<(unsigned)blocks, threads, 0, st>>>(p, pos, dir, pol, time, wavelength);
+    const uint64_t blocks = (p.n + kSampleThreads - 1) / kSampleThreads;
+    k_sample_source<<<(unsigned)blocks, kSampleThreads, 0, st>>>(p, pos, dir, pol, time, wavelength);
     return cudaGetLastError();
 }
 
