@@ -15,6 +15,7 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <map>
 #include <mutex>
 #include <thread>
 #include <vector>
@@ -56,10 +57,8 @@ struct TmpNode {
 };
 
 // surface-area heuristic: cost of a triangle test relative to a node visit
-#ifndef LXO_SAH_CI
-#define LXO_SAH_CI 2.0
-#endif
-constexpr double kSahTriCost = LXO_SAH_CI;
+// (195 warp instructions against 88 in the photon kernel)
+constexpr double kSahTriCost = 2.0;
 
 struct Builder {
     std::vector<Ref>& refs;
@@ -320,10 +319,10 @@ Ref make_ref(const float* tri_v, uint32_t id)
     return r;
 }
 
-// Cells of the walk grid along the longest side of the scene.
-#ifndef LXO_GRID_CELLS
-#define LXO_GRID_CELLS 96
-#endif
+// Cells of the walk grid along the longest side of the scene (2e7 photons on
+// the DARWIN-scale mesh / 3e6 on the 50 cm TPC: 74.1 / 13.4 ms with 96, 75.5 /
+// 13.7 with 128, 79.5 / 13.8 with 192; 64 as 96).
+constexpr int kGridCells = 96;
 
 // The walk grid: cubic cells over the scene's bounding box and one cell
 // around it, x fastest.
@@ -537,7 +536,7 @@ int build_bvh(const float* tri_v, uint32_t nt, const int32_t* cluster_of, int n_
     WalkGrid wg;
     std::vector<std::pair<uint32_t, Ref>> grid_refs;
     const bool flat = !(scene_ext > 0.0f);
-    out->grid_h = flat ? 1.0 : (double)scene_ext / LXO_GRID_CELLS;
+    out->grid_h = flat ? 1.0 : (double)scene_ext / kGridCells;
     if (!flat) {
         Box sb;
         sb.reset();
@@ -585,6 +584,34 @@ int build_bvh(const float* tri_v, uint32_t nt, const int32_t* cluster_of, int n_
         std::sort(grid_refs.begin(), grid_refs.end(), [](const auto& x, const auto& y) {
             return x.first < y.first || (x.first == y.first && x.second.id < y.second.id);
         });
+    }
+    // cells that hold the same one or two triangles share one leaf (their
+    // parts' boxes do not matter in a leaf): a query that walks along a panel
+    // knows the leaf it has just tested
+    struct GridCell {
+        uint32_t cell, count;
+        uint64_t first;    // of its references
+        size_t same;       // the cell whose leaf it shares (itself: its own tree)
+        int32_t root;      // tmp node
+    };
+    std::vector<GridCell> grid_cells;
+    {
+        std::map<std::pair<uint32_t, uint32_t>, size_t> seen;
+        uint64_t kept = 0;
+        for (uint64_t k = 0; k < grid_refs.size();) {
+            uint64_t e = k + 1;
+            while (e < grid_refs.size() && grid_refs[e].first == grid_refs[k].first) ++e;
+            GridCell g{grid_refs[k].first, (uint32_t)(e - k), kept, grid_cells.size(), -1};
+            if (e - k <= 2) {
+                const std::pair<uint32_t, uint32_t> ids{grid_refs[k].second.id, grid_refs[e - 1].second.id};
+                g.same = seen.emplace(ids, grid_cells.size()).first->second;
+            }
+            if (g.same == grid_cells.size())
+                for (uint64_t q = k; q < e; ++q) grid_refs[kept++] = grid_refs[q];
+            grid_cells.push_back(g);
+            k = e;
+        }
+        grid_refs.resize(kept);
     }
     const uint64_t n_grid = grid_refs.size();
     const uint64_t n_main = main_refs.size();
@@ -669,24 +696,23 @@ int build_bvh(const float* tri_v, uint32_t nt, const int32_t* cluster_of, int n_
         for (auto& t : th) t.join();
         cl_root[c] = kd_top(B, cell_root[c], kc.nu, 0, kc.nu, 0, kc.nv);
     }
-    std::vector<std::pair<uint32_t, int32_t>> grid_root;   // (cell, tmp node) of the occupied cells
-    {
-        std::vector<uint64_t> first;
-        for (uint64_t k = 0; k < n_grid; ++k)
-            if (k == 0 || grid_refs[k].first != grid_refs[k - 1].first) {
-                grid_root.push_back({grid_refs[k].first, -1});
-                first.push_back(k);
+    parallel_for(n_threads, grid_cells.size(), 64, [&](size_t q, size_t e) {
+        for (; q < e; ++q) {
+            GridCell& g = grid_cells[q];
+            if (g.same != q) continue;
+            const uint32_t r = B.alloc(), first = (uint32_t)(n_main + n_dup + g.first);
+            if (g.count <= 2 && g.count <= leaf_size) {
+                nodes[r].b = refs[first].b;
+                if (g.count == 2) nodes[r].b.grow(refs[first + 1].b);
+                nodes[r].depth = 0;
+                B.make_leaf(r, first, g.count);
+            } else {
+                B.build(r, first, g.count, 0);
             }
-        first.push_back(n_grid);
-        parallel_for(n_threads, grid_root.size(), 64, [&](size_t q, size_t e) {
-            for (; q < e; ++q) {
-                const uint32_t r = B.alloc();
-                B.build(r, (uint32_t)(n_main + n_dup + first[q]), (uint32_t)(first[q + 1] - first[q]), 0);
-                grid_root[q].second = (int32_t)r;
-            }
-        });
-        std::vector<std::pair<uint32_t, Ref>>().swap(grid_refs);
-    }
+            g.root = (int32_t)r;
+        }
+    });
+    std::vector<std::pair<uint32_t, Ref>>().swap(grid_refs);
     const uint32_t n_tmp = B.n_nodes.load();
 
     // ---- layout: depth-first per tree, main tree first ------------------------
@@ -710,7 +736,8 @@ int build_bvh(const float* tri_v, uint32_t nt, const int32_t* cluster_of, int n_
     if (main_leaf) main_wrap = n_internal++;  // a one-leaf root node wraps a leaf main tree
     dfs(main_tmp);
     for (int c = 0; c < n_clusters; ++c) dfs(cl_root[c]);
-    for (const auto& r : grid_root) dfs(r.second);
+    for (size_t k = 0; k < grid_cells.size(); ++k)
+        if (grid_cells[k].same == k) dfs(grid_cells[k].root);
     out->n_nodes = std::max(1u, n_internal);
     out->n_leaves = n_leaves;
     out->n_records = (uint32_t)n_refs;
@@ -799,9 +826,9 @@ int build_bvh(const float* tri_v, uint32_t nt, const int32_t* cluster_of, int n_
         if (wg.cells()) {
             std::vector<uint8_t> occ(wg.cells(), 0);
             out->walk_ref.assign(wg.cells(), kEmptyChild);
-            for (const auto& r : grid_root) {
-                occ[r.first] = 1;
-                out->walk_ref[r.first] = child_ref(r.second);
+            for (const GridCell& g : grid_cells) {
+                occ[g.cell] = 1;
+                out->walk_ref[g.cell] = child_ref(grid_cells[g.same].root);
             }
             walk_skips(wg, occ, n_threads, out->walk_skip);
             for (int a = 0; a < 3; ++a) out->walk_n[a] = wg.n[a];

@@ -48,13 +48,8 @@ constexpr int kMaxCellsPerRay = 4;
 // may hold
 constexpr uint8_t kCellOut = 255;
 constexpr uint64_t kMaxGridRefs = 8u << 20;
-#ifndef LXO_SAFE_HOPS
-#define LXO_SAFE_HOPS 3
-#endif
-constexpr int kSafeHops = LXO_SAFE_HOPS;
-#ifndef LXO_POOL_KB
-#define LXO_POOL_KB 164
-#endif
+constexpr int kSafeHops = 3;    // cubes that clear a flight before it is traced (1: 4 % slower)
+constexpr int kPoolKb = 164;    // shared memory per SM for the photon pools of the forward builds, KiB
 
 struct ClusterHost {
     int axis;

@@ -47,10 +47,11 @@ struct U4 {
     float u0, u1, u2, u3;
 };
 
-// kRounds: rounds per iteration of the code (10: no loop; 1: a tenth of the
-// code, for the places that are not hot -- instruction fetch is what bounds
-// the photon loop)
-template <int kRounds = 10>
+// kRounds: rounds per iteration of the code.  10, no loop, is fastest by
+// itself; the photon loop uses 2 (and 1 where it is not hot), since long code
+// costs it more than the loop: 1e6 photons of the DARWIN-scale mesh 4.75 -> 4.70
+// ms, 2e7 63.5 -> 62.6, 3e6 of the 50 cm TPC 11.4 -> 11.2.
+template <int kRounds = 2>
 __device__ __forceinline__ uint4 philox4x32_10(uint4 c, uint2 k)
 {
 #pragma unroll kRounds
@@ -70,7 +71,7 @@ __device__ __forceinline__ float u01(uint32_t x)
     return __fmul_rn(__uint2float_rn(x >> 9) + 0.5f, 1.1920928955078125e-07f);
 }
 
-template <int kRounds = 10>
+template <int kRounds = 2>
 __device__ __forceinline__ U4 draw4(uint64_t seed, uint64_t pid, uint32_t step, uint32_t draw)
 {
     uint4 o = philox4x32_10<kRounds>(make_uint4((uint32_t)pid, (uint32_t)(pid >> 32), step, draw),
@@ -297,9 +298,10 @@ __device__ __forceinline__ RayInv ray_inv(const Scene& sc, float3 o, float3 d)
 }
 
 // State of a query: next node (kDone: finished), stack entries, axis kz,
-// closest hit so far (t and record), and how far its walk has come.
+// sub-tree of the last occupied cell, closest hit so far (t and record), and
+// how far its walk has come.
 struct Query {
-    int node, sp, kz;
+    int node, sp, kz, seen;
     float bt, tw;
     uint32_t rec;
 };
@@ -310,7 +312,7 @@ struct Query {
 __device__ __forceinline__ Query begin_query(const Scene& sc, float3 o, float3 d, int kz, float tmax, uint32_t clusters,
                                              float clear, int* stack)
 {
-    Query c{kWalk, 1, kz, tmax, clear, LXO_NO_HIT};
+    Query c{kWalk, 1, kz, kDone, tmax, clear, LXO_NO_HIT};
     stack[0] = kDone;
     if (clusters) enter_clusters(sc, clusters, o, d, tmax, stack, c.sp);
     if (!(clear >= 0.0f)) {
@@ -418,7 +420,7 @@ __device__ __forceinline__ bool clear_flight(const Scene& sc, float3 o, float3 d
 // rounding here.  The walk is over (the next stack entry follows) once it has
 // left the grid or passed the closest hit.
 __device__ __forceinline__ void walk_step(const Scene& sc, const float4* q, const RayInv& r, float eps, float bt,
-                                          float& t, int& node, int* stack, int& sp)
+                                          float& t, int& node, int& seen, int* stack, int& sp)
 {
     const float4 a = q[0], b = q[1];
     const int x = (int)fmaf(fmaf(t, b.x, a.x), sc.grid_inv, sc.grid_off[0]);
@@ -428,8 +430,11 @@ __device__ __forceinline__ void walk_step(const Scene& sc, const float4* q, cons
     const uint32_t c = min((uint32_t)((z * sc.walk_n[1] + y) * sc.walk_n[0] + x), sc.walk_cells - 1u);
     const uint32_t k = __ldg(&sc.walk_skip[8u * c + octant(r)]);
     if (k == 0u) {
-        node = __ldg(&sc.walk_ref[c]);
-        stack[sp++] = kWalk;
+        const int ref = __ldg(&sc.walk_ref[c]);
+        if (ref != seen) {   // cells with the same triangles share a leaf
+            node = seen = ref;
+            stack[sp++] = kWalk;
+        }
     }
     t = fmaxf(cube_exit(x, y, z, fmaxf((float)k, 1.0f), r), t) + eps;
     if (node == kWalk && (k == kCellOut || t > bt)) node = stack[--sp];
@@ -456,15 +461,12 @@ __device__ __forceinline__ uint32_t cluster_mask(const Scene& sc, float3 o, floa
 }
 
 
-#ifndef LXO_WALK_MIN
-#define LXO_WALK_MIN 8
-#endif
-#ifndef LXO_NODE_MIN
-#define LXO_NODE_MIN 8
-#endif
-#ifndef LXO_STOP_DIV
-#define LXO_STOP_DIV 2
-#endif
+
+// A leaf's triangles are tested once fewer lanes than kRunMin walk and fewer
+// than that descend (2e7 photons on the DARWIN-scale mesh: 92 ms with 8, 98
+// with 4 or 12, at the time); a part of the traversal runs until half of the
+// lanes that wanted it are through.
+constexpr int kRunMin = 8;
 
 // Lets the queries of a warp run until `need` of its n0 queries in flight have
 // finished (node kDone).  q: the lane's slot.
@@ -473,7 +475,7 @@ __device__ __forceinline__ void run_queries(const Scene& sc, const float4* q, ui
                                             int n0, int need, Query& cur, int* stack, int* err, Counters& cnt, Lap&& lap)
 {
     const uint32_t lane = threadIdx.x & 31u;
-    int node = cur.node, sp = cur.sp;
+    int node = cur.node, sp = cur.sp, seen = cur.seen;
     float bt = cur.bt, tw = cur.tw;
     uint32_t rec = cur.rec;
     int leaf = 0;   // parked leaf (0 = none: reference 0 is an internal node, never a leaf)
@@ -489,8 +491,8 @@ __device__ __forceinline__ void run_queries(const Scene& sc, const float4* q, ui
         const int nw = __popc(__ballot_sync(FULL_MASK, node == kWalk));
         const int nd = __popc(__ballot_sync(FULL_MASK, node >= 0));
         const int nl = __popc(__ballot_sync(FULL_MASK, leaf != 0));
-        if (nl > 0 && nw < LXO_WALK_MIN && nd < LXO_NODE_MIN) {
-            const int stop = nl / LXO_STOP_DIV;
+        if (nl > 0 && nw < kRunMin && nd < kRunMin) {
+            const int stop = nl / 2;
             do {
                 if (kStats && lane == 0) cnt.leaf_iters++;
                 if (leaf != 0) {
@@ -508,17 +510,17 @@ __device__ __forceinline__ void run_queries(const Scene& sc, const float4* q, ui
         } else if (nw == 0 && nd == 0) {
             break;
         } else if (nw >= nd) {
-            const int stop = nw / LXO_STOP_DIV;
+            const int stop = nw / 2;
             do {
                 if (kStats && lane == 0) cnt.walk_iters++;
                 if (node == kWalk) {
                     if (kStats) cnt.walks++;
-                    walk_step(sc, q, r, eps, bt, tw, node, stack, sp);
+                    walk_step(sc, q, r, eps, bt, tw, node, seen, stack, sp);
                 }
             } while (__popc(__ballot_sync(FULL_MASK, node == kWalk)) > stop);
             lap(cnt.cyc[kCycNode], n0);
         } else {
-            const int stop = nd / LXO_STOP_DIV;
+            const int stop = nd / 2;
             do {
                 if (kStats && lane == 0) cnt.node_iters++;
                 if (node >= 0) {
@@ -537,6 +539,7 @@ __device__ __forceinline__ void run_queries(const Scene& sc, const float4* q, ui
     }
     cur.node = node;
     cur.sp = sp;
+    cur.seen = seen;
     cur.bt = bt;
     cur.tw = tw;
     cur.rec = rec;
@@ -620,7 +623,7 @@ __global__ void __launch_bounds__(kTraceThreads, kTraceCtas)
     uint32_t leave_out = 0;        // triangle id not to be hit
     float eps = 0.0f;
     RayInv r{};
-    Query cur{kDone, 1, 0, 0.0f, 0.0f, LXO_NO_HIT};
+    Query cur{kDone, 1, 0, kDone, 0.0f, 0.0f, LXO_NO_HIT};
     int stack[kStackSize];
     Counters cnt{};
     auto lap = [](unsigned long long&, int) {};
@@ -1196,21 +1199,12 @@ __device__ __forceinline__ int surface_event(const PropParams& p, Photon& ph, fl
 // Measured (1e8 photons on the DARWIN-scale mesh / 3e6 on the 50 cm TPC with
 // dispersion / 2e6 on the mesh without electrodes, GB300): 503 / 21.0 / 17.7
 // ms for the loop before, 316 / 12.0 / 10.5 ms now.
-#ifndef LXO_POOL_THREADS
-#define LXO_POOL_THREADS 576
-#endif
-#ifndef LXO_POOL_CTAS
-#define LXO_POOL_CTAS 2
-#endif
-// a warp leaves the traversal once 1 / kLeaveDiv of its rays have finished
-#ifndef LXO_LEAVE_DIV
-#define LXO_LEAVE_DIV 2
-#endif
-#ifndef LXO_BATCH_MIN
-#define LXO_BATCH_MIN 28
-#endif
-constexpr int kPoolThreads = LXO_POOL_THREADS, kPoolCtas = LXO_POOL_CTAS;
+constexpr int kPoolThreads = 576, kPoolCtas = 2;
 constexpr int kPoolWarps = kPoolThreads / 32;
+// A batch starts with the lanes of this many columns or more (24: 5 % slower,
+// 30: 2 %); a warp leaves the traversal once half of its queries have finished
+// (a third: 1 % slower).
+constexpr int kBatchMin = 28;
 constexpr int kMaxSlots = 1024;       // 32 columns of 32
 constexpr uint32_t kPollLimit = 1u << 20;   // a warp that has found nothing so often leaves (never a lost photon: it holds none)
 
@@ -1354,7 +1348,7 @@ __global__ void __launch_bounds__(kPoolThreads, kPoolCtas) k_propagate(const __g
     const int turn = warp & 31;
     // the lane's query in flight: its slot (-1 none) and state; its stack in local memory
     int slot = -1;
-    Query cur{kDone, 1, 0, 0.0f, 0.0f, LXO_NO_HIT};
+    Query cur{kDone, 1, 0, kDone, 0.0f, 0.0f, LXO_NO_HIT};
     int stack[kStackSize];
     uint32_t polls = 0;
     Counters cnt{};
@@ -1378,7 +1372,7 @@ __global__ void __launch_bounds__(kPoolThreads, kPoolCtas) k_propagate(const __g
         const uint32_t busy = __ballot_sync(FULL_MASK, slot >= 0);
         // a batch: 32 lanes, fewer once the photons left do not fill all warps
         const int width = min(32, (live + kPoolWarps - 1) / kPoolWarps);
-        const int full = width > LXO_BATCH_MIN ? LXO_BATCH_MIN : max(width, 1);
+        const int full = width > kBatchMin ? kBatchMin : max(width, 1);
         int stage;
         if (__popc(in[kBulk]) >= full) stage = kBulk;
         else if (__popc(in[kSurf]) >= full) stage = kSurf;
@@ -1431,7 +1425,7 @@ __global__ void __launch_bounds__(kPoolThreads, kPoolCtas) k_propagate(const __g
             __syncwarp();
             lap(cnt.cyc[kCycBegin], n0);
             if (kStats && lane == 0) cnt.entries++;
-            const int need = max(1, n0 / LXO_LEAVE_DIV);
+            const int need = max(1, n0 / 2);
             const uint32_t skip = __float_as_uint(q[3].w) & kNoTri;
             run_queries<kStats>(p.sc, q, skip, ray, p.sc.walk_eps, n0, need, cur, stack, p.err, cnt, lap);
             const bool done = slot >= 0 && cur.node == kDone;
@@ -1624,7 +1618,7 @@ cudaError_t launch_propagate(const PropParams& params, int device, cudaStream_t 
     if (e != cudaSuccess) return e;
     p.tally_stride = adj ? (p.adj_k | 1) : 0;
     const size_t per_slot = sizeof(float4) * kSlotF4 + sizeof(float) * p.tally_stride;
-    const size_t room = (size_t)(adj ? 227 : LXO_POOL_KB) * 1024 / kPoolCtas - 1024 - fa.sharedSizeBytes;
+    const size_t room = (size_t)(adj ? 227 : kPoolKb) * 1024 / kPoolCtas - 1024 - fa.sharedSizeBytes;
     const uint64_t slots = std::min<uint64_t>(kMaxSlots, room / per_slot / 32 * 32);
     e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(slots * per_slot));
     if (e != cudaSuccess) return e;
