@@ -222,12 +222,15 @@ typedef struct {
     unsigned long long* stats;   /* device [LXO_STATS_LEN] with LXO_FLAG_STATS (accumulated): [0..3]
                                     photon steps, BVH nodes visited, leaves visited, triangles tested
                                     (lane counts); [4..6] warp iterations of the node loop, of the
-                                    leaf loop and of the photon loop; [7..8] lane cycles in
-                                    traversal, in steps; [9..17] steps in material 0 by nodes
-                                    visited (bins of 8, last >= 64), [18] their leaves; [19..28]
-                                    the same for other materials; [29..34] lane cycles in the node
-                                    loop, the leaf loop, the traversal set-up, the step's draws, the
-                                    interaction, and the refill (tallies, new photons) */
+                                    leaf loop and batches of steps; [7..8] lane cycles (a warp's
+                                    clock times the lanes at work) in traversal, in all; [9..17]
+                                    steps in material 0 by nodes visited (bins of 8, last >= 64),
+                                    [18] their leaves; [19..28] the same for other materials;
+                                    [29..34] lane cycles in walk and node loop, the leaf loop, the
+                                    traversal set-up, the next step's draws and flight, the
+                                    interaction, and the refill (tallies, new photons); [35]
+                                    entries into the traversal, [36] lane cycles without work,
+                                    [37..38] steps of the walk, its warp iterations */
     float* ph_state;             /* optional device [n*9]: per photon, its state when it met its fate
                                     (or was cut by max_steps): position (mm), unit direction and unit
                                     polarisation, 3 floats each -- so the outgoing wave of every

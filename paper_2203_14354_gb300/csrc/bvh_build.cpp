@@ -16,7 +16,9 @@
 #include <cstdlib>
 #include <cstring>
 #include <map>
+#include <memory>
 #include <mutex>
+#include <new>
 #include <thread>
 #include <vector>
 
@@ -337,13 +339,20 @@ template <class F>
 void parallel_for(uint32_t n_threads, size_t n, size_t grain, F&& body)   // body(first, last) over [0, n)
 {
     std::atomic<size_t> next{0};
+    std::atomic<bool> failed{false};   // an exception stays in its thread
     auto work = [&]() {
-        for (size_t i = next.fetch_add(grain); i < n; i = next.fetch_add(grain)) body(i, std::min(n, i + grain));
+        try {
+            for (size_t i = next.fetch_add(grain); i < n && !failed.load(); i = next.fetch_add(grain))
+                body(i, std::min(n, i + grain));
+        } catch (...) {
+            failed.store(true);
+        }
     };
     std::vector<std::thread> th;
     for (uint32_t t = 1; t < std::min<size_t>(n_threads, (n + grain - 1) / grain); ++t) th.emplace_back(work);
     work();
     for (auto& t : th) t.join();
+    if (failed.load()) throw std::bad_alloc();
 }
 
 // Cells that triangle v may touch, each once: a triangle whose box (widened
@@ -664,6 +673,7 @@ int build_bvh(const float* tri_v, uint32_t nt, const int32_t* cluster_of, int n_
 
     // ---- trees ----------------------------------------------------------------
     TmpNode* nodes = (TmpNode*)malloc(sizeof(TmpNode) * (2ull * n_refs + 4ull * 16e6 + 8));
+    const std::unique_ptr<TmpNode, void (*)(void*)> nodes_owner(nodes, free);
     if (!nodes) {
         snprintf(err, err_len, "build_bvh: out of host memory");
         return -1;
@@ -748,7 +758,6 @@ int build_bvh(const float* tri_v, uint32_t nt, const int32_t* cluster_of, int n_
     for (int c = 0; c < n_clusters; ++c) n_cells += (uint32_t)cl[c].cell_count.size();
     out->cells = (int32_t*)malloc(sizeof(int32_t) * std::max(1u, n_cells));
     if (!out->nodes || !out->tris || !out->cells) {
-        free(nodes);
         free_bvh(out);
         snprintf(err, err_len, "build_bvh: out of host memory");
         return -1;
@@ -822,24 +831,16 @@ int build_bvh(const float* tri_v, uint32_t nt, const int32_t* cluster_of, int n_
         cell_off += (uint32_t)kc.cell_count.size();
     }
     out->n_cells = cell_off;
-    try {
-        if (wg.cells()) {
-            std::vector<uint8_t> occ(wg.cells(), 0);
-            out->walk_ref.assign(wg.cells(), kEmptyChild);
-            for (const GridCell& g : grid_cells) {
-                occ[g.cell] = 1;
-                out->walk_ref[g.cell] = child_ref(grid_cells[g.same].root);
-            }
-            walk_skips(wg, occ, n_threads, out->walk_skip);
-            for (int a = 0; a < 3; ++a) out->walk_n[a] = wg.n[a];
+    if (wg.cells()) {
+        std::vector<uint8_t> occ(wg.cells(), 0);
+        out->walk_ref.assign(wg.cells(), kEmptyChild);
+        for (const GridCell& g : grid_cells) {
+            occ[g.cell] = 1;
+            out->walk_ref[g.cell] = child_ref(grid_cells[g.same].root);
         }
-    } catch (...) {
-        free(nodes);
-        free_bvh(out);
-        snprintf(err, err_len, "build_bvh: out of host memory");
-        return -1;
+        walk_skips(wg, occ, n_threads, out->walk_skip);
+        for (int a = 0; a < 3; ++a) out->walk_n[a] = wg.n[a];
     }
-    free(nodes);
     out->sah_cost = sah;
     out->build_seconds = std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
     return 0;

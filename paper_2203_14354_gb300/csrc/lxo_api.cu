@@ -415,11 +415,16 @@ lxo_status lxo_build_bvh(lxo_ctx* c, const lxo_bvh_params* bp, lxo_bvh_info* inf
     const float expand = std::ldexp(c->max_abs, -19);
     // thin dense layers (electrode wire meshes, PMT arrays) get their own
     // grid-entered trees
-    std::vector<int32_t> cluster_of(c->nt, -1);
-    const int n_clusters = lxo::detect_layers(c->tri_v.data(), c->nt, cluster_of.data());
-    if (lxo::build_bvh(c->tri_v.data(), c->nt, cluster_of.data(), n_clusters, q.leaf_size, q.sah_bins, q.n_threads,
-                       expand, &b, msg, sizeof msg))
-        return fail(c, LXO_ERR_NOMEM, "%s", msg);
+    try {
+        std::vector<int32_t> cluster_of(c->nt, -1);
+        const int n_clusters = lxo::detect_layers(c->tri_v.data(), c->nt, cluster_of.data());
+        if (lxo::build_bvh(c->tri_v.data(), c->nt, cluster_of.data(), n_clusters, q.leaf_size, q.sah_bins, q.n_threads,
+                           expand, &b, msg, sizeof msg))
+            return fail(c, LXO_ERR_NOMEM, "%s", msg);
+    } catch (...) {
+        lxo::free_bvh(&b);
+        return fail(c, LXO_ERR_NOMEM, "build_bvh: out of host memory");
+    }
     // attributes of each record
     for (uint32_t k = 0; k < b.n_records; ++k) {
         float4& r2 = b.tris[3ull * k + 2];

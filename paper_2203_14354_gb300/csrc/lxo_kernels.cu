@@ -1,6 +1,6 @@
 // Device code of the photon tracker (sm_103a).
 //
-//  * k_trace:          one ray per lane, closest hit (the geometry query alone).
+//  * k_trace, k_trace_few: closest hits of given rays (the geometry query alone).
 //  * k_sample_source:  first photon state from a source (one photon per lane).
 //  * k_propagate:      persistent kernel; the photons of a CTA wait in slots in
 //                      shared memory for one of four kinds of work (query of
@@ -602,7 +602,7 @@ __global__ void k_trace_few(const __grid_constant__ Scene sc, const float* __res
 // from which its lanes take their next ray when half of those in flight have
 // finished.  What bounds it is the divergence of the queries (a lane a ray to
 // the end of the warp's slowest, whole trees searched: 397 us for 2e6 rays
-// with free-flight limits in the DARWIN-scale mesh; now 251 us).
+// with free-flight limits in the DARWIN-scale mesh; now 240 us).
 constexpr int kTraceThreads = 128, kTraceCtas = 9, kTraceWarps = kTraceThreads / 32, kTraceRing = 64;
 
 __global__ void __launch_bounds__(kTraceThreads, kTraceCtas)
@@ -1011,8 +1011,6 @@ __device__ __forceinline__ void spawn_offset(Photon& ph, float3 o_ray, float t_h
     ph.pos = ph.pos + (side * eps) * N;
 }
 
-// one interaction; returns -1 if the photon lives on, else its fate code
-// (detail set to channel / material / surface / triangle)
 // First half of a step: the step's uniforms and the absorption / Rayleigh
 // distances in the current medium.
 struct StepDraw {
@@ -1182,7 +1180,7 @@ __device__ __forceinline__ int surface_event(const PropParams& p, Photon& ph, fl
 // is issue slots times lanes at work: the loop this replaced kept a photon in
 // a lane for its whole life and ran every kind of work for the few lanes that
 // needed it (9.3 lanes of 32 per instruction, 210 instructions per photon
-// step of a warp; here 17.3 and 114).  The draws of the next step and its
+// step of a warp; here 18.3 and 103).  The draws of the next step and its
 // flight's set-up belong to the batch that ends the step before, with all
 // lanes at work.
 // Flights that meet nothing need no query: the walk grid's empty cubes clear
@@ -1191,22 +1189,30 @@ __device__ __forceinline__ int surface_event(const PropParams& p, Photon& ph, fl
 // Instruction fetch is what is left: the requests that miss the SM's
 // instruction cache came at the same 0.515 per cycle and GPC in three versions
 // of this loop, so hot code is kept short (82 KB -> 75 KB: 8 to 12 % less
-// time).
+// time).  So does the length of each warp's own chain: 20 instructions more in
+// the choice of the next batch cost 3 to 7 %.
 // Launch shape: CTAs of kPoolThreads threads, kPoolCtas per SM: 18 warps of 56
 // registers each; 2e7 photons on the DARWIN-scale mesh / 3e6 on the 50 cm TPC
 // took 63.1 / 11.4 ms, with 2 x 640 threads of 48 registers 66.5 / 12.0, with
 // 2 x 512 of 64 66.8 / 11.4, with 3 x 384 of 56 66.4 / 11.4.
 // Measured (1e8 photons on the DARWIN-scale mesh / 3e6 on the 50 cm TPC with
 // dispersion / 2e6 on the mesh without electrodes, GB300): 503 / 21.0 / 17.7
-// ms for the loop before, 316 / 12.0 / 10.5 ms now.
+// ms for the loop before, 305 / 11.5 / 10.0 ms now.
 constexpr int kPoolThreads = 576, kPoolCtas = 2;
 constexpr int kPoolWarps = kPoolThreads / 32;
 // A batch starts with the lanes of this many columns or more (24: 5 % slower,
 // 30: 2 %); a warp leaves the traversal once half of its queries have finished
 // (a third: 1 % slower).
 constexpr int kBatchMin = 28;
+// The last photons of a CTA are shared out: a batch takes at most 1 / kSpread of
+// them, so that a photon's step does not wait for those of all others (3e5
+// photons of the mesh without electrodes: 3.39 ms with 8, 3.61 with 18, the
+// warps of the CTA, 4.29 with 30; 3e5 of the 50 cm TPC 2.70 / 2.87 / 3.29).
+constexpr int kSpread = 8;
 constexpr int kMaxSlots = 1024;       // 32 columns of 32
-constexpr uint32_t kPollLimit = 1u << 20;   // a warp that has found nothing so often leaves (never a lost photon: it holds none)
+// a warp that has found nothing so often leaves (it holds no photon; the
+// others go on with theirs)
+constexpr uint32_t kPollLimit = 1u << 20;
 
 // Where a slot's photon waits.
 enum { kReady = 0, kReadyLayer, kBulk, kSurf, kFree, kSets };
@@ -1370,8 +1376,8 @@ __global__ void __launch_bounds__(kPoolThreads, kPoolCtas) k_propagate(const __g
         for (int k = 0; k < kSets; ++k) in[k] = __ballot_sync(FULL_MASK, *(volatile uint32_t*)&s_set[k][lane] != 0u);
         const int live = __shfl_sync(FULL_MASK, *(volatile int*)&s_live, 0);
         const uint32_t busy = __ballot_sync(FULL_MASK, slot >= 0);
-        // a batch: 32 lanes, fewer once the photons left do not fill all warps
-        const int width = min(32, (live + kPoolWarps - 1) / kPoolWarps);
+        // a batch: 32 lanes, fewer once few photons are left
+        const int width = min(32, (live + kSpread - 1) / kSpread);
         const int full = width > kBatchMin ? kBatchMin : max(width, 1);
         int stage;
         if (__popc(in[kBulk]) >= full) stage = kBulk;
