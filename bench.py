@@ -42,14 +42,14 @@ OPS_PER_NODE, OPS_PER_TRI, OPS_PHYSICS = 40, 50, 250
 N_SM, LANES_PER_SM = 152, 128
 # DRAM bytes (read + write) per photon of the propagation kernel: ncu
 # dram__bytes_read.sum + dram__bytes_write.sum of one timed launch on 2e6
-# photons of this workload (8.423 GB + 4.602 GB), divided by 2e6; scales with
-# the photon count.  Most of the writes, and a third of the reads, are the
-# 32-register build's spills and traversal stack leaving L1 and L2.
-DRAM_BYTES_PER_PHOTON = 6512
+# photons of this workload (5.447 GB + 0.261 GB), divided by 2e6; scales with
+# the photon count.  Nearly all of it reads nodes and triangle records of the
+# wire meshes.
+DRAM_BYTES_PER_PHOTON = 2854
 # warp instructions issued per photon step by the same capture
-# (smsp__inst_executed.sum 1.0792e10 over 5.147e7 steps); the issue-slot peak
+# (smsp__inst_executed.sum 5.923e9 over 5.147e7 steps); the issue-slot peak
 # is 152 SMs x 4 schedulers x 1 warp instruction per cycle x the SM clock
-WARP_INST_PER_STEP = 209.7
+WARP_INST_PER_STEP = 115.1
 SCHEDULERS_PER_SM = 4
 # The kernel build those two numbers were captured from: its ptxas
 # signature and the SHA-256 of its sources.  When the built kernel differs,
@@ -57,8 +57,8 @@ SCHEDULERS_PER_SM = 4
 # be taken again).
 TIMED_KERNEL = "_ZN3lxo11k_propagateILb0ELb0ELb0EEEvNS_10PropParamsE"   # k_propagate<0,0,0>
 KERNEL_SOURCES = ("paper_2203_14354_gb300/csrc/lxo_kernels.cu", "paper_2203_14354_gb300/csrc/lxo_internal.h")
-CAPTURED_KERNEL = {"registers": 32, "spill_stores": 538, "spill_loads": 616,
-                   "sources_sha256": "1fa675c8893873eba0ba098175fb9ad1a31d29e08863aa4f1dad41da785a8a8a"}
+CAPTURED_KERNEL = {"registers": 56, "spill_stores": 88, "spill_loads": 48,
+                   "sources_sha256": "c0aef295cb49e45921083440beef039b7ede4358ce8f1cee02af154b82d28f4d"}
 
 
 def parse():
@@ -192,8 +192,8 @@ def adjoint_cost(args, n=10_000_000, reps=3):
     """Forward + adjoint against the plain forward on the 50 cm TPC with 61 +
     61 PMTs and thin-disk electrodes, 1e7 photons, 7 parameters: the time of
     the propagation with per-photon tallies (and the Jacobian kernel) over the
-    time of the plain propagation, same photons, each at its faster register
-    budget (5 or 8 CTAs of 256 threads per SM)."""
+    time of the plain propagation, same photons, each at the faster of two
+    launch shapes (5 or 8 CTAs of 256 threads per SM)."""
     import torch
     from paper_2203_14354_gb300 import geometry, Tracker
     det = geometry.scaled_tpc()
