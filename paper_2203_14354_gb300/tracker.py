@@ -343,8 +343,9 @@ class Tracker:
         return out
 
     def set_launch(self, blocks_per_sm=0, chunk=0, threads=0):
-        """Launch shape: CTAs per SM (0 = occupancy limit), photon ids per
-        warp grab (0 = 64), threads per CTA (128 or 256; 0 = 256)."""
+        """Launch shape: blocks_per_sm CTAs of `threads` (128 or 256; 0 = 256)
+        limit the threads on each SM (0 = no limit); chunk limits the photon
+        ids that a warp takes at once (0 = 64; it takes at most 32)."""
         self._check(self._L.lxo_set_launch(self._ctx, blocks_per_sm, chunk, threads))
 
 
