@@ -594,9 +594,12 @@ int build_bvh(const float* tri_v, uint32_t nt, const int32_t* cluster_of, int n_
             return x.first < y.first || (x.first == y.first && x.second.id < y.second.id);
         });
     }
-    // cells that hold the same one or two triangles share one leaf (their
-    // parts' boxes do not matter in a leaf): a query that walks along a panel
-    // knows the leaf it has just tested
+    // cells that hold the same one or two triangles share one leaf: a query
+    // that walks along a panel knows the leaf it has just tested.  It has to be
+    // a leaf (no more triangles than leaf_size): the parts' boxes, which are
+    // those of the first cell, do not matter in a leaf, but an inner node would
+    // test every other cell's ray against them
+    const uint64_t share_max = std::min(2u, leaf_size);
     struct GridCell {
         uint32_t cell, count;
         uint64_t first;    // of its references
@@ -611,7 +614,7 @@ int build_bvh(const float* tri_v, uint32_t nt, const int32_t* cluster_of, int n_
             uint64_t e = k + 1;
             while (e < grid_refs.size() && grid_refs[e].first == grid_refs[k].first) ++e;
             GridCell g{grid_refs[k].first, (uint32_t)(e - k), kept, grid_cells.size(), -1};
-            if (e - k <= 2) {
+            if (e - k <= share_max) {
                 const std::pair<uint32_t, uint32_t> ids{grid_refs[k].second.id, grid_refs[e - 1].second.id};
                 g.same = seen.emplace(ids, grid_cells.size()).first->second;
             }
@@ -711,7 +714,7 @@ int build_bvh(const float* tri_v, uint32_t nt, const int32_t* cluster_of, int n_
             GridCell& g = grid_cells[q];
             if (g.same != q) continue;
             const uint32_t r = B.alloc(), first = (uint32_t)(n_main + n_dup + g.first);
-            if (g.count <= 2 && g.count <= leaf_size) {
+            if (g.count <= share_max) {
                 nodes[r].b = refs[first].b;
                 if (g.count == 2) nodes[r].b.grow(refs[first + 1].b);
                 nodes[r].depth = 0;
