@@ -326,6 +326,13 @@ Ref make_ref(const float* tri_v, uint32_t id)
 // 13.7 with 128, 79.5 / 13.8 with 192; 64 as 96).
 constexpr int kGridCells = 96;
 
+// The margin by which triangles reach over their cells, in cells: kMinPad, or
+// four times that of the node boxes, which grows with the coordinates.  Where
+// that comes to more than kMaxPad (coordinates of more than 341 times the
+// scene's size), every cell would hold most of its neighbours' triangles, and
+// there is no grid.
+constexpr double kMinPad = 0.01, kMaxPad = 0.25;
+
 // The walk grid: cubic cells over the scene's bounding box and one cell
 // around it, x fastest.
 struct WalkGrid {
@@ -357,7 +364,9 @@ void parallel_for(uint32_t n_threads, size_t n, size_t grain, F&& body)   // bod
 
 // Cells that triangle v may touch, each once: a triangle whose box (widened
 // by the pad) spans more than two cells along an axis is halved across its
-// longest edge until its parts' boxes do not.
+// longest edge until its parts' boxes do not.  (That comes to an end because
+// the pad is at most a quarter of a cell, see kMaxPad: parts of half a cell
+// span two cells at most.)
 void touched_cells(const WalkGrid& g, const float* v, std::vector<uint32_t>& out)
 {
     double t[64][3][3];   // parts still to do
@@ -540,21 +549,23 @@ int build_bvh(const float* tri_v, uint32_t nt, const int32_t* cluster_of, int n_
         else split_refs(&tri_v[9ull * i], i, r.b, max_ext, 0, main_refs);
     }
     // walk grid: the main-tree triangles again, each in every cell that it
-    // touches, by its part inside the cell (both widened by the pad, 1 % of a
-    // cell); left out (kept empty) if that takes more than kMaxGridRefs parts
+    // touches, by its part inside the cell (both widened by the pad); left out
+    // (kept empty) if that takes more than kMaxGridRefs parts, or if the pad
+    // would be too large
     WalkGrid wg;
     std::vector<std::pair<uint32_t, Ref>> grid_refs;
     const bool flat = !(scene_ext > 0.0f);
     out->grid_h = flat ? 1.0 : (double)scene_ext / kGridCells;
-    if (!flat) {
-        Box sb;
-        sb.reset();
-        for (uint64_t k = 0; k < 3ull * nt; ++k) sb.grow(&tri_v[3 * k]);
+    Box sb;
+    sb.reset();
+    for (uint64_t k = 0; !flat && k < 3ull * nt; ++k) sb.grow(&tri_v[3 * k]);
+    for (int a = 0; !flat && a < 3; ++a) out->grid_org[a] = (double)sb.lo[a] - out->grid_h;
+    if (!flat && 4.0 * (double)expand <= kMaxPad * out->grid_h) {
         wg.h = out->grid_h;
-        wg.pad = std::max(0.01 * wg.h, 4.0 * (double)expand);
+        wg.pad = std::max(kMinPad * wg.h, 4.0 * (double)expand);
         for (int a = 0; a < 3; ++a) {
             wg.n[a] = std::max(1, (int)std::ceil(((double)sb.hi[a] - sb.lo[a]) / wg.h)) + 2;
-            wg.org[a] = out->grid_org[a] = (double)sb.lo[a] - wg.h;
+            wg.org[a] = out->grid_org[a];
         }
         std::vector<uint32_t> ids;
         for (uint32_t i = 0; i < nt; ++i)
@@ -586,7 +597,7 @@ int build_bvh(const float* tri_v, uint32_t nt, const int32_t* cluster_of, int n_
             std::lock_guard<std::mutex> lock(mu);
             grid_refs.insert(grid_refs.end(), part.begin(), part.end());
         });
-        if (total.load() > kMaxGridRefs) {
+        if (total.load() > kMaxGridRefs || main_refs.size() + n_dup + total.load() >= (1ull << 28)) {
             std::vector<std::pair<uint32_t, Ref>>().swap(grid_refs);
             wg = WalkGrid();
         }

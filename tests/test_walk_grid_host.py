@@ -2,12 +2,17 @@
 point of a triangle lies in, the search meets that triangle.  Points are drawn
 in double and rounded to float, off the plane by far less than the margin of
 the boxes (2^-19 of the largest coordinate, 32 float steps of it)."""
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 
 from paper_2203_14354_gb300 import geometry as g
 from tests.cuda.host import walk_grid_check
 
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 DETECTORS = {
     "box": lambda: g.reflector_box(),                 # 12 triangles over thousands of cells
     "soup": lambda: g.random_soup(3000, seed=5, extent=60.0, size=15.0),
@@ -30,3 +35,30 @@ def test_every_point_is_found_from_its_cell(name, leaf_size):
     pts, ids = points(det, 40_000, seed=leaf_size)
     status, lost, seen = walk_grid_check(det, pts, ids, leaf_size)
     assert status == 1 and seen == len(ids) and lost == 0
+
+
+# a mesh of 4 mm at `offset` mm: the grid's margin grows with the coordinates, up to a quarter of a cell at 341
+# times the mesh's size; beyond that there is no grid
+FAR_MESH = """
+import sys
+sys.path.insert(0, {root!r})
+from tests.test_walk_grid_host import far_sphere, points, walk_grid_check
+det = far_sphere({offset})
+print(walk_grid_check(det, *points(det, 20_000, seed=1)))
+"""
+
+
+def far_sphere(offset):
+    det = g.icosphere(2.0, 2)   # 320 triangles
+    det.verts = (det.verts.astype(np.float64) + [0.0, 0.0, offset]).astype(np.float32)
+    return det
+
+
+@pytest.mark.parametrize("offset, grid", [(0.0, 1), (-100.0, 1), (-1300.0, 1), (-2600.0, 0), (-3000.0, 0), (2e6, 0)])
+def test_small_mesh_far_from_the_origin(offset, grid):
+    # (in a process of its own, which can be ended: a build that splits triangles without end does not return)
+    r = subprocess.run([sys.executable, "-c", FAR_MESH.format(root=ROOT, offset=offset)], capture_output=True,
+                       text=True, timeout=60)
+    assert r.returncode == 0, r.stderr[-2000:]
+    status, lost, seen = eval(r.stdout)
+    assert status == grid and lost == 0 and seen == (20_000 if grid else 0)
