@@ -1626,7 +1626,9 @@ cudaError_t launch_propagate(const PropParams& params, int device, cudaStream_t 
     const size_t per_slot = sizeof(float4) * kSlotF4 + sizeof(float) * p.tally_stride;
     const size_t room = (size_t)(adj ? 227 : kPoolKb) * 1024 / kPoolCtas - 1024 - fa.sharedSizeBytes;
     const uint64_t slots = std::min<uint64_t>(kMaxSlots, room / per_slot / 32 * 32);
-    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(slots * per_slot));
+    // the kernel's limit is one value for all threads of the process: the room,
+    // which does not depend on this launch's tallies
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)room);
     if (e != cudaSuccess) return e;
     int per_sm = 0;
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kPoolThreads, slots * per_slot);
