@@ -183,9 +183,14 @@ struct Builder {
         nodes[idx].count = 0;
         const uint32_t big = 1u << 16;
         if (count > big && threads_free.fetch_sub(1) > 0) {
-            std::thread t([=] { build(l, first, nl, depth + 1); });
+            std::thread t;
+            try {
+                t = std::thread([=] { build(l, first, nl, depth + 1); });
+            } catch (...) {   // no thread to be had
+                build(l, first, nl, depth + 1);
+            }
             build(r, first + nl, count - nl, depth + 1);
-            t.join();
+            if (t.joinable()) t.join();
             threads_free.fetch_add(1);
         } else {
             if (count > big) threads_free.fetch_add(1);
@@ -356,7 +361,10 @@ void parallel_for(uint32_t n_threads, size_t n, size_t grain, F&& body)   // bod
         }
     };
     std::vector<std::thread> th;
-    for (uint32_t t = 1; t < std::min<size_t>(n_threads, (n + grain - 1) / grain); ++t) th.emplace_back(work);
+    try {
+        for (uint32_t t = 1; t < std::min<size_t>(n_threads, (n + grain - 1) / grain); ++t) th.emplace_back(work);
+    } catch (...) {   // as many as there are to be had
+    }
     work();
     for (auto& t : th) t.join();
     if (failed.load()) throw std::bad_alloc();
@@ -705,19 +713,12 @@ int build_bvh(const float* tri_v, uint32_t nt, const int32_t* cluster_of, int n_
         if (kc.n == 0) continue;
         const size_t ncell = kc.cell_count.size();
         cell_root[c].assign(ncell, -1);
-        std::atomic<size_t> next{0};
-        auto work = [&]() {
-            for (size_t q = next.fetch_add(1); q < ncell; q = next.fetch_add(1)) {
-                if (!kc.cell_count[q]) continue;
-                const uint32_t r = B.alloc();
-                B.build(r, kc.cell_first[q], kc.cell_count[q], 0);
-                cell_root[c][q] = (int32_t)r;
-            }
-        };
-        std::vector<std::thread> th;
-        for (uint32_t t = 1; t < n_threads; ++t) th.emplace_back(work);
-        work();
-        for (auto& t : th) t.join();
+        parallel_for(n_threads, ncell, 1, [&](size_t q, size_t) {
+            if (!kc.cell_count[q]) return;
+            const uint32_t r = B.alloc();
+            B.build(r, kc.cell_first[q], kc.cell_count[q], 0);
+            cell_root[c][q] = (int32_t)r;
+        });
         cl_root[c] = kd_top(B, cell_root[c], kc.nu, 0, kc.nu, 0, kc.nv);
     }
     parallel_for(n_threads, grid_cells.size(), 64, [&](size_t q, size_t e) {

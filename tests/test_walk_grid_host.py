@@ -62,3 +62,26 @@ def test_small_mesh_far_from_the_origin(offset, grid):
     assert r.returncode == 0, r.stderr[-2000:]
     status, lost, seen = eval(r.stdout)
     assert status == grid and lost == 0 and seen == (20_000 if grid else 0)
+
+
+# no thread can be started (a default stack larger than the address space): the build does with its own
+NO_THREADS = """
+import ctypes, sys
+sys.path.insert(0, {root!r})
+from tests.test_walk_grid_host import DETECTORS, g, points, walk_grid_check
+det = g.icosphere(2.0, 7)   # 327680 triangles: trees and grid are shared out over threads
+pts = points(det, 20_000, seed=1)
+walk_grid_check(DETECTORS["box"](), *points(DETECTORS["box"](), 10, seed=1))   # compiled before the threads go
+libc, attr = ctypes.CDLL(None), ctypes.create_string_buffer(256)
+assert libc.pthread_attr_init(attr) == 0
+assert libc.pthread_attr_setstacksize(attr, ctypes.c_size_t(1 << 47)) == 0
+assert libc.pthread_setattr_default_np(attr) == 0
+print(walk_grid_check(det, *pts, n_threads=8))
+"""
+
+
+def test_build_without_threads():
+    r = subprocess.run([sys.executable, "-c", NO_THREADS.format(root=ROOT)], capture_output=True, text=True,
+                       timeout=120)
+    assert r.returncode == 0, r.stderr[-2000:]
+    assert eval(r.stdout) == (1, 0, 20_000)
