@@ -420,13 +420,21 @@ __device__ __forceinline__ bool clear_flight(const Scene& sc, float3 o, float3 d
 // rounding here.  The walk is over (the next stack entry follows) once it has
 // left the grid or passed the closest hit.
 __device__ __forceinline__ void walk_step(const Scene& sc, const float4* q, const RayInv& r, float eps, float bt,
-                                          float& t, int& node, int& seen, int* stack, int& sp)
+                                          float& t, int& node, int& seen, int* stack, int& sp, int* err)
 {
     const float4 a = q[0], b = q[1];
     const int x = (int)fmaf(fmaf(t, b.x, a.x), sc.grid_inv, sc.grid_off[0]);
     const int y = (int)fmaf(fmaf(t, b.y, a.y), sc.grid_inv, sc.grid_off[1]);
     const int z = (int)fmaf(fmaf(t, b.z, a.z), sc.grid_inv, sc.grid_off[2]);
-    // (inside the grid by construction; the limit guards the memory)
+    // inside the grid by construction, which the checked build compares; the
+    // limit guards the memory in the other
+    if (LXO_CHECK_BOUNDS && ((uint32_t)x >= (uint32_t)sc.walk_n[0] || (uint32_t)y >= (uint32_t)sc.walk_n[1] ||
+                             (uint32_t)z >= (uint32_t)sc.walk_n[2])) {
+        atomicOr(err, kErrBounds);
+        node = kDone;
+        sp = 1;
+        return;
+    }
     const uint32_t c = min((uint32_t)((z * sc.walk_n[1] + y) * sc.walk_n[0] + x), sc.walk_cells - 1u);
     const uint32_t k = __ldg(&sc.walk_skip[8u * c + octant(r)]);
     if (k == 0u) {
@@ -515,7 +523,7 @@ __device__ __forceinline__ void run_queries(const Scene& sc, const float4* q, ui
                 if (kStats && lane == 0) cnt.walk_iters++;
                 if (node == kWalk) {
                     if (kStats) cnt.walks++;
-                    walk_step(sc, q, r, eps, bt, tw, node, seen, stack, sp);
+                    walk_step(sc, q, r, eps, bt, tw, node, seen, stack, sp, err);
                 }
             } while (__popc(__ballot_sync(FULL_MASK, node == kWalk)) > stop);
             lap(cnt.cyc[kCycNode], n0);
