@@ -188,12 +188,11 @@ def cpu_baseline(det, target_s):
                       f"scene build excluded"}, res, n
 
 
-def adjoint_cost(args, n=10_000_000, reps=3):
+def adjoint_cost(args, n=10_000_000, reps=5):
     """Forward + adjoint against the plain forward on the 50 cm TPC with 61 +
     61 PMTs and thin-disk electrodes, 1e7 photons, 7 parameters: the time of
     the propagation with per-photon tallies (and the Jacobian kernel) over the
-    time of the plain propagation, same photons, each at the faster of two
-    launch shapes (5 or 8 CTAs of 256 threads per SM)."""
+    time of the plain propagation, same photons."""
     import torch
     from paper_2203_14354_gb300 import geometry, Tracker
     det = geometry.scaled_tpc()
@@ -209,29 +208,23 @@ def adjoint_cost(args, n=10_000_000, reps=3):
         if adj:
             trk.jacobian(out["adjoint"])
 
-    times, shapes, table = {}, {}, {}
+    times = {}
     for adj in (False, True):
-        for bps in (5, 8):
-            trk.set_launch(bps, 0, 256)
+        run(adj)
+        trk.sync()
+        ts = []
+        for _ in range(reps):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
             run(adj)
-            trk.sync()
-            ts = []
-            for _ in range(reps):
-                a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
-                a.record()
-                run(adj)
-                b.record()
-                torch.cuda.synchronize()
-                ts.append(a.elapsed_time(b))
-            table[f"{'adjoint' if adj else 'forward'} {bps} CTAs/SM"] = statistics.median(ts)
-            if adj not in times or statistics.median(ts) < times[adj]:
-                times[adj], shapes[adj] = statistics.median(ts), bps
-    trk.set_launch(0, 0, 0)
+            b.record()
+            torch.cuda.synchronize()
+            ts.append(a.elapsed_time(b))
+        times[adj] = statistics.median(ts)
     trk.sync()
     res = {"workload": "50 cm dual-phase TPC, 61+61 PMTs, thin-disk gate/anode/cathode, 1e7 photons, 7 parameters",
            "fwd_ms": times[False], "fwd_adjoint_ms": times[True], "ratio": times[True] / times[False],
-           "fwd_photons_per_s": n / (times[False] / 1e3),
-           "ctas_per_sm": {"forward": shapes[False], "adjoint": shapes[True]}, "ms_by_shape": table}
+           "fwd_photons_per_s": n / (times[False] / 1e3)}
     if not args.no_adjoint_fd:
         res["fd_check"] = adjoint_fd_check(trk)
     return res
@@ -457,7 +450,7 @@ def events_throughput(det, reps=3):
     trk.upload_events(ev[::10])
     sub = trk.alloc_event_results(256, hist=False)
     best, table = autotune_launch(trk, lambda: trk.propagate_events(seed=1, out=sub, hist=False, sync=False),
-                                  blocks=(5, 6, 8), chunks=(32, 64, 128), threads=(128, 256), reps=2)
+                                  blocks=(2, 5), chunks=(16, 32), reps=2)
     del sub
     trk.upload_events(ev)
     out = trk.alloc_event_results(256, hist=True)

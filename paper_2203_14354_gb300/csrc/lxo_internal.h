@@ -194,9 +194,9 @@ struct PropParams {
     uint32_t first_event;              // event id of events[0]: photon ids ((first_event + e) << 32) | i
     const EventDev* events;            // [n_events]
     const unsigned long long* ev_prefix;  // [n_events + 1] photon-count prefix sums
-    uint32_t chunk;                    // photon ids per warp grab
-    uint32_t blocks_per_sm;            // 0 = occupancy limit
-    uint32_t block_threads;            // threads per CTA of the propagation kernel: 128 or 256 (0 = 256)
+    uint32_t chunk;                    // most photon ids that a warp takes at once (32 at most in any case)
+    uint32_t blocks_per_sm;            // with block_threads, the threads that a launch may keep on each SM
+    uint32_t block_threads;            //   (rounded up to whole CTAs of the kernel); 0 = no limit
     int slots, tally_stride;     // photon slots per CTA, floats of adjoint tallies per slot (set by the launch)
     unsigned long long* queue;   // scratch: work-queue head
     int* err;                    // scratch: device error word

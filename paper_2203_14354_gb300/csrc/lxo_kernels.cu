@@ -493,8 +493,6 @@ __device__ __forceinline__ uint32_t cluster_mask(const Scene& sc, float3 o, floa
     return m;
 }
 
-
-
 // A leaf's triangles are tested once fewer lanes than kRunMin walk and fewer
 // than that descend (2e7 photons on the DARWIN-scale mesh: 92 ms with 8, 98
 // with 4 or 12, at the time); a part of the traversal runs until half of the
@@ -529,10 +527,8 @@ __device__ __forceinline__ void run_queries(const Scene& sc, const float4* q, ui
             do {
                 if (kStats && lane == 0) cnt.leaf_iters++;
                 if (leaf != 0) {
-                    {
                     const float4 o = q[0], sh = q[4];   // origin and shear constants wait in the slot
                     triangle(sc, WRay{o.x, o.y, o.z, sh.x, sh.y, sh.z, cur.kz}, skip, leaf, bt, rec, err);
-                }
                     if (kStats) {
                         cnt.q_leaves += leaf == 0;
                         cnt.tris++;
@@ -581,7 +577,16 @@ __device__ __forceinline__ void run_queries(const Scene& sc, const float4* q, ui
 // ---------------------------------------------------------------------------
 // rays given by the caller
 // ---------------------------------------------------------------------------
-// fewer rays than this: k_trace_few
+// Fewer rays than this: k_trace_few.  Time of k_trace_few over that of k_trace,
+// rays without / with free-flight limits:
+//                          1e5 rays      2e5           4e5           8e5
+//   small TPC              0.82 / 0.90   1.14 / 1.17   1.37 / 1.39   1.59 / 1.61
+//   50 cm TPC              1.13 / 0.92   1.29 / 1.19   1.44 / 1.47   1.64 / 1.77
+//   3000 loose triangles   1.12 / 1.04   1.53 / 1.55   1.81 / 1.88   2.18 / 2.14
+//   box of 16 triangles    0.52 / 0.56   0.81 / 0.80   1.00 / 0.95   1.19 / 1.20
+//   DARWIN-scale mesh      0.80 / 0.81   0.89 / 0.88   0.96 / 0.98   1.06 / 1.26
+//   the same, wires        0.68 / 0.73   0.80 / 0.75   0.97 / 0.92   1.09 / 1.16
+// The line lies where the last of them break even, within 8 %.
 constexpr uint32_t kTraceMany = 400000;
 // Few rays: one lane a ray to its end through layers and main tree.  Little
 // code, which is what counts when the kernel lasts as long as a few hundred
@@ -634,9 +639,11 @@ __global__ void k_trace_few(const __grid_constant__ Scene sc, const float* __res
 // Many rays.  A warp looks at 32 rays at a time: those whose whole flight the empty cubes
 // clear are answered at once, the others wait in a ring of the warp's own,
 // from which its lanes take their next ray when half of those in flight have
-// finished.  What bounds it is the divergence of the queries (a lane a ray to
-// the end of the warp's slowest, whole trees searched: 397 us for 2e6 rays
-// with free-flight limits in the DARWIN-scale mesh; now 240 us).
+// finished.  What bounds it is the wait for nodes and triangles (60 % of a
+// warp's cycles; L1 hits 40 %, L2 52 %, DRAM 13 % in use), with 15.8 of 32 lanes
+// at work, and the last rays (an SM is busy for some 80 % of the time).  2e6 rays
+// with free-flight limits in the DARWIN-scale mesh: 240 us, 397 with a lane a
+// ray to the end of the warp's slowest and whole trees searched.
 constexpr int kTraceThreads = 128, kTraceCtas = 9, kTraceWarps = kTraceThreads / 32, kTraceRing = 64;
 
 __global__ void __launch_bounds__(kTraceThreads, kTraceCtas)
@@ -763,9 +770,6 @@ __device__ __forceinline__ bool inside_poly(const SourceDev& s, float x, float y
     return x * s.side_cos[k] + y * s.side_sin[k] <= s.apothem;
 }
 
-// Event of global photon index idx (binary search on the prefix sums) and
-// the photon's first state: direction and polarisation as for any source,
-// position from the event's point / segment / ball.
 // Emission delay of the scintillation time profile (Sec. 2.2, Table 2): a
 // mixture of two exponentials, from its own draw of the source step.
 __device__ __forceinline__ float emission_delay(const U4& u, const TimeProfile& tp)
@@ -809,6 +813,9 @@ __device__ __forceinline__ U4 emission_draw(const PropParams& p, uint64_t pid, c
     return draw4<kRounds>(p.seed, pid, kSourceStep, 0xFFFFFFFFu);
 }
 
+// Event of global photon index idx (binary search on the prefix sums) and
+// the photon's first state: direction and polarisation as for any source,
+// position from the event's point / segment / ball.
 // kRounds: see philox4x32_10; want_wl: the wavelength is wanted.
 template <int kRounds>
 __device__ Photon make_event_photon(const PropParams& p, uint64_t idx, bool want_wl)
@@ -921,10 +928,14 @@ __device__ Photon make_photon(const PropParams& p, uint64_t idx, bool want_wl)
     return ph;
 }
 
-// Bound by issue slots (three generator calls, six sines and cosines, two
-// logarithms a photon), so the stores are plain: through shared memory, in full
-// lines, 4e6 photons with time profile and spectrum took 98 us, so 90 before
-// the two emission draws became one and 84 now.
+// 588 instructions a photon (three generator calls, six sines and cosines, two
+// logarithms) would be 58 us for 4e6 photons at one a cycle and scheduler; it
+// takes 84, with 69 % of the issue slots in use.  In the others no warp is ready:
+// they wait for busy pipes (the one for indexed constants, the sides of the
+// polygon, 64 %, integer 51 %) and for results of the special functions.  The
+// stores are plain, since they are not what it waits for (LSU 6 % in use, DRAM
+// 17 %): through shared memory, in full lines, the kernel took 98 us, with 90
+// before the two emission draws became one and 84 now.
 constexpr int kSampleThreads = 128;
 
 __global__ void k_sample_source(const __grid_constant__ PropParams p, float* pos, float* dir, float* pol,
@@ -1046,10 +1057,10 @@ __device__ __forceinline__ void spawn_offset(Photon& ph, float3 o_ray, float t_h
     ph.pos = ph.pos + (side * eps) * N;
 }
 
-// First half of a step: the step's uniforms and the absorption / Rayleigh
-// distances in the current medium.
+// First half of a step: the absorption / Rayleigh distances in the current
+// medium (the first two uniforms of the step's draw).
 struct StepDraw {
-    float d_abs, d_ray, u2, u3;
+    float d_abs, d_ray;
 };
 
 template <bool kSpectral>
@@ -1069,13 +1080,8 @@ __device__ __forceinline__ StepDraw begin_step(const PropParams& p, const Photon
     // of the adjoint tallies to see it (measured, 2 % faster)
     sd.d_abs = isinf(mt.abs_len) ? INFINITY : -mt.abs_len * logf(u.u0);
     sd.d_ray = isinf(ray_len) ? INFINITY : -ray_len * logf(u.u1);
-    sd.u2 = u.u2;
-    sd.u3 = u.u3;
     return sd;
 }
-
-
-
 
 // Second half of a step that met no surface: bulk absorption or Rayleigh
 // scattering at the sampled distance d_int (absorbed: the absorption distance
@@ -1215,7 +1221,7 @@ __device__ __forceinline__ int surface_event(const PropParams& p, Photon& ph, fl
 // is issue slots times lanes at work: the loop this replaced kept a photon in
 // a lane for its whole life and ran every kind of work for the few lanes that
 // needed it (9.3 lanes of 32 per instruction, 210 instructions per photon
-// step of a warp; here 18.3 and 103).  The draws of the next step and its
+// step of a warp; here 17.6 and 115).  The draws of the next step and its
 // flight's set-up belong to the batch that ends the step before, with all
 // lanes at work.
 // Flights that meet nothing need no query: the walk grid's empty cubes clear
@@ -1234,7 +1240,6 @@ __device__ __forceinline__ int surface_event(const PropParams& p, Photon& ph, fl
 // dispersion / 2e6 on the mesh without electrodes, GB300): 503 / 21.0 / 17.7
 // ms for the loop before, 305 / 11.5 / 10.0 ms now.
 constexpr int kPoolThreads = 576, kPoolCtas = 2;
-constexpr int kPoolWarps = kPoolThreads / 32;
 // A batch starts with the lanes of this many columns or more (24: 5 % slower,
 // 30: 2 %); a warp leaves the traversal once half of its queries have finished
 // (a third: 1 % slower).

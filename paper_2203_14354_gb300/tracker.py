@@ -349,30 +349,37 @@ class Tracker:
         self._check(self._L.lxo_set_launch(self._ctx, blocks_per_sm, chunk, threads))
 
 
+POOL_THREADS, POOL_CTAS = 576, 2   # shape of the photon kernel: threads per CTA, CTAs per SM
+
+
 def autotune_launch(tracker, run, blocks=(2, 3, 4, 5), chunks=(32, 64, 128, 256), threads=(256,), reps=2):
     """Times `run()` (one launch of the workload to tune, on the current
     stream) for every launch shape (threads per CTA x CTAs per SM x chunk;
     CTAs per SM are counted in 256-thread units, so 128-thread CTAs run
     twice as many) and keeps the fastest; returns (threads, blocks_per_sm,
     chunk, ms) and the table of timings keyed by (threads, blocks_per_sm,
-    chunk)."""
-    table = {}
+    chunk).  Shapes that come to the same launch of the photon kernel (whole
+    CTAs per SM, 32 ids at most) are timed once and share their time."""
+    table, timed = {}, {}
     for t in threads:
         for b in blocks:
             for c in chunks:
                 bps = b * (256 // t)
-                tracker.set_launch(bps, c, t)
-                run()
-                torch.cuda.synchronize()
-                ts = []
-                for _ in range(reps):
-                    e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
-                    e0.record()
+                launch = (min(POOL_CTAS, -(-bps * t // POOL_THREADS)) if bps else POOL_CTAS, min(c or 64, 32))
+                if launch not in timed:
+                    tracker.set_launch(bps, c, t)
                     run()
-                    e1.record()
                     torch.cuda.synchronize()
-                    ts.append(e0.elapsed_time(e1))
-                table[(t, bps, c)] = min(ts)
+                    ts = []
+                    for _ in range(reps):
+                        e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+                        e0.record()
+                        run()
+                        e1.record()
+                        torch.cuda.synchronize()
+                        ts.append(e0.elapsed_time(e1))
+                    timed[launch] = min(ts)
+                table[(t, bps, c)] = timed[launch]
     best = min(table, key=table.get)
     tracker.set_launch(best[1], best[2], best[0])
     return (*best, table[best]), table
